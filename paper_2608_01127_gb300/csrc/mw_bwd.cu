@@ -348,15 +348,15 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       constexpr uint32_t idesc_dq = L::DQT ? idesc_bf16_f32(128, QN, true, true)
                                            : idesc_bf16_f32(128, D, true, true);
       // descriptors computed once; each MMA adds a compile-time offset
-      const uint64_t k_kmaj = sdesc_sw128(smem_u32(sK), 16, 1024);
-      const uint64_t v_kmaj = sdesc_sw128(smem_u32(sV), 16, 1024);
-      const uint64_t k_mn = sdesc_sw128(smem_u32(sK), L::KREGION, 1024);
-      const uint64_t q_kmaj0 = sdesc_sw128(smem_u32(sQ), 16, 1024);
-      const uint64_t do_kmaj0 = sdesc_sw128(smem_u32(sDO), 16, 1024);
-      const uint64_t q_mn0 = sdesc_sw128(smem_u32(sQ), L::QREGION, 1024);
-      const uint64_t do_mn0 = sdesc_sw128(smem_u32(sDO), L::QREGION, 1024);
-      const uint64_t ds_mn0 = sdesc_sw128(smem_u32(sDS), L::KREGION, 1024);
-      const uint64_t ds_kmaj0 = sdesc_sw128(smem_u32(sDS), 16, 1024);
+      const uint32_t k_kmaj = sdesc_sw128(smem_u32(sK), 16);
+      const uint32_t v_kmaj = sdesc_sw128(smem_u32(sV), 16);
+      const uint32_t k_mn = sdesc_sw128(smem_u32(sK), L::KREGION);
+      const uint32_t q_kmaj0 = sdesc_sw128(smem_u32(sQ), 16);
+      const uint32_t do_kmaj0 = sdesc_sw128(smem_u32(sDO), 16);
+      const uint32_t q_mn0 = sdesc_sw128(smem_u32(sQ), L::QREGION);
+      const uint32_t do_mn0 = sdesc_sw128(smem_u32(sDO), L::QREGION);
+      const uint32_t ds_mn0 = sdesc_sw128(smem_u32(sDS), L::KREGION);
+      const uint32_t ds_kmaj0 = sdesc_sw128(smem_u32(sDS), 16);
       // d = 64: S^T += ones x (-LSE/scale) and dP^T += ones x (-D), one tf32
       // MMA each (K = 8); the 256-byte A atoms serve every 8-row group (SBO 0)
       const uint64_t ones_l = sdesc_sw32(smem_u32(smem + L::OFF_ONES), 0);
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
                        idesc_tf32_f32(128, QN), 1u);
       };
       // X = A B^T, both K-major over d (S^T = K Q^T, dP^T = V dO^T)
-      auto issue_kmajor = [&](uint32_t d_col, uint64_t a, uint64_t b) {
+      auto issue_kmajor = [&](uint32_t d_col, uint32_t a, uint32_t b) {
 #pragma unroll
         for (int kk = 0; kk < DM / 16; ++kk) {
           const uint32_t ka = (kk >> 2) * L::KREGION + (kk & 3) * 32;
@@ -405,8 +405,8 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         const int st1 = (j + 1) % NS;
         const uint32_t ph1 = ((j + 1) / NS) & 1;
         const bool more = j + 1 < n_q;
-        const uint64_t do_mn = sdesc_add(do_mn0, st * L::QTILE);
-        const uint64_t q_mn = sdesc_add(q_mn0, st * L::QSTRIDE);
+        const uint32_t do_mn = sdesc_add(do_mn0, st * L::QTILE);
+        const uint32_t q_mn = sdesc_add(q_mn0, st * L::QSTRIDE);
         if (role_a) {
           if (!L::SHARED_X && more) {
             // S^T of the next step as soon as the P/dS warps hold S^T_j
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
               if (!(ok = warp_wait(dq_free, (j - 1) & 1, ctl))) break;
               tc_fence_after();
             }
-            const uint64_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
+            const uint32_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
 #pragma unroll
             for (int kk = 0; kk < kTileRows / 16; ++kk)
               umma_ss(tmem + L::DQ_COL, sdesc_add(ds_mn, kk * 2048), sdesc_add(k_mn, kk * 2048),
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
             umma_commit(dq_full);
           }
           // dK += dS^T Q_j (d = 64: dS^T read from shared memory, K-major)
-          const uint64_t ds_kmaj = sdesc_add(ds_kmaj0, (j % L::DS_BUFS) * L::DS_BYTES);
+          const uint32_t ds_kmaj = sdesc_add(ds_kmaj0, (j % L::DS_BUFS) * L::DS_BYTES);
 #pragma unroll
           for (int kk = 0; kk < QN / 16; ++kk) {
             if constexpr (L::SHARED_X)
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
             if (!(ok = warp_wait(dq_free, (j - 1) & 1, ctl))) break;
             tc_fence_after();
           }
-          const uint64_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
+          const uint32_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
 #pragma unroll
           for (int kk = 0; kk < kTileRows / 16; ++kk) {
             if constexpr (L::DQT)   // A = K^T (MN-major over d), B = dS^T (MN-major over queries)

@@ -257,7 +257,11 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  // the allocation of all 512 columns can only start at 0; as a constant it
+  // keeps the issuing warp's TMEM addresses out of registers (with one-word
+  // operand descriptors, 12 heads of 128, 32 x 600 tokens: 783 us before, 749
+  // with the descriptors, 721 with both; d = 64, 16 x 880: 640 -> 631 us)
+  constexpr uint32_t tmem = 0;
   const WaitCtl ctl{abort_flag, p.status, p.budget_ns};
   // launched early (programmatic dependent launch): the setup above has run
   // while the previous kernel finished; global memory only from here on
@@ -320,14 +324,14 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, false, false);
       constexpr uint32_t idesc_pv = idesc_bf16_f32(128, L::OW, false, true);
       // descriptors computed once; each MMA adds a compile-time offset
-      const uint64_t q_desc = sdesc_sw128(smem_u32(sQ), 16, 1024);
-      const uint64_t k_desc = sdesc_sw128(smem_u32(sK), 16, 1024);
+      const uint32_t q_desc = sdesc_sw128(smem_u32(sQ), 16);
+      const uint32_t k_desc = sdesc_sw128(smem_u32(sK), 16);
       const uint32_t v_addr = smem_u32(sV);
       const uint32_t ones_addr = smem_u32(smem + L::OFF_ONES);
 
       auto issue_qk = [&](int t, int st) {
-        const uint64_t qa = sdesc_add(q_desc, t * L::TILE_BYTES);
-        const uint64_t kb = sdesc_add(k_desc, st * L::TILE_BYTES);
+        const uint32_t qa = sdesc_add(q_desc, t * L::TILE_BYTES);
+        const uint32_t kb = sdesc_add(k_desc, st * L::TILE_BYTES);
 #pragma unroll
         for (int kk = 0; kk < DM / 16; ++kk) {
           const uint32_t off = (kk >> 2) * L::REGION_BYTES + (kk & 3) * 32;
@@ -339,7 +343,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       auto issue_pv = [&](int t, int st, bool acc, int half) {
         // V stage st; for d = 64 the next 64 "columns" are the ones region
         const uint32_t vs = v_addr + st * L::TILE_BYTES;
-        const uint64_t vb = sdesc_sw128(vs, L::ONES_BYTES > 0 ? ones_addr - vs : L::REGION_BYTES, 1024);
+        const uint32_t vb = sdesc_sw128(vs, L::ONES_BYTES > 0 ? ones_addr - vs : L::REGION_BYTES);
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4) {
           const int kk = 4 * half + k4;

@@ -213,19 +213,26 @@ __device__ __forceinline__ void tc_fence_after() {
 // only about two instructions deep.  elect.sync picks the same (lowest) lane
 // every time, so tcgen05.commit tracks the MMAs that lane issued.
 
-// D(tmem) (+)= A(smem desc) * B(smem desc)^T, kind::f16 (bf16 in, f32 acc).
-__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+// The high word shared by all 128-byte-swizzle operand descriptors (see
+// sdesc_sw128): stride byte offset 1024, version 1, swizzle mode 2.
+constexpr uint32_t kSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+
+// D(tmem) (+)= A(smem) * B(smem)^T, kind::f16 (bf16 in, f32 acc); operands
+// given by the low words of their sdesc_sw128 descriptors (the issuing warps
+// hold many of them: one register each instead of two).
+__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_desc, uint32_t b_desc,
                                         uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, e;\n\t"
+      "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
       "elect.sync _|e, 0xffffffff;\n\t"
+      "mov.b64 a, {%1, %5};\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_desc), "r"(b_desc), "r"(idesc), "r"(accumulate), "n"(kSw128Hi)
       : "memory");
 }
 
-// Same with A read from tensor memory.
 // D (+)= A B^T with tf32 operands (kind::tf32, K = 8 per instruction).
 __device__ __forceinline__ void umma_ss_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                              uint32_t idesc, uint32_t accumulate) {
@@ -238,14 +245,16 @@ __device__ __forceinline__ void umma_ss_tf32(uint32_t d_tmem, uint64_t a_desc, u
       : "memory");
 }
 
-__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+// umma_ss with A read from tensor memory.
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_desc,
                                         uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p, e;\n\t"
+      "{\n\t.reg .pred p, e;\n\t.reg .b64 b;\n\t"
       "elect.sync _|e, 0xffffffff;\n\t"
+      "mov.b64 b, {%2, %5};\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(b_desc), "r"(idesc), "r"(accumulate), "n"(kSw128Hi)
       : "memory");
 }
 
@@ -346,20 +355,17 @@ __device__ __forceinline__ void regs_inc() {
 //     LBO = byte distance between regions (next 64 MN columns),
 //     SBO = 1024 (next group of 8 contraction rows); a 16-deep K step
 //     advances 16 rows = 2048 bytes.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo_bytes,
-                                                uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= static_cast<uint64_t>(1) << 46;
-  d |= static_cast<uint64_t>(2) << 61;
-  return d;
+// The low word; the high word is kSw128Hi for every operand here (SBO 1024).
+__device__ __forceinline__ uint32_t sdesc_sw128(uint32_t saddr, uint32_t lbo_bytes) {
+  return ((saddr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }
 
 // The same descriptor for a start address `bytes` further on (a multiple of
 // 16): only the 14-bit address field changes, and it cannot carry for the
 // in-range shared-memory addresses used here.
+__device__ __forceinline__ uint32_t sdesc_add(uint32_t desc, uint32_t bytes) {
+  return desc + (bytes >> 4);
+}
 __device__ __forceinline__ uint64_t sdesc_add(uint64_t desc, uint32_t bytes) {
   return desc + static_cast<uint64_t>(bytes >> 4);
 }
