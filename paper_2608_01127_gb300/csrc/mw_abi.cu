@@ -119,14 +119,15 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 // 3-D map over [BH, rows, d] with the 128-byte swizzle the tcgen05
 // descriptors and the drain's boxes use; rows past the end read as zero.
-// bf16 operands: 64-column x box_rows boxes.  f32 (the dQ accumulator):
-// 32-column x box_rows boxes.
+// bf16 operands: 64-column x box_rows boxes.  f32 (split partials, the dQ
+// accumulator): 32-column x box_rows boxes.  cols: the columns of a row that
+// exist for the copies (the rest of its d are neither read nor written).
 mw_status encode_map(CUtensorMap* m, const void* ptr, int rows, int BH, int d, const char* name,
-                     int box_rows, bool f32 = false) {
+                     int box_rows, bool f32, int cols) {
   auto fn = encode_fn();
   if (!fn) return fail(MW_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable (no CUDA driver?)");
   const cuuint64_t es = f32 ? 4 : 2;
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(rows),
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows),
                         static_cast<cuuint64_t>(BH)};
   cuuint64_t strides[2] = {static_cast<cuuint64_t>(d) * es,
                            static_cast<cuuint64_t>(rows) * d * es};
@@ -147,9 +148,10 @@ struct MapKey {
   const void* ptr;
   int rows, BH, d, box_rows;
   bool f32;
+  int cols;
   bool operator==(const MapKey& o) const {
     return ptr == o.ptr && rows == o.rows && BH == o.BH && d == o.d && box_rows == o.box_rows &&
-           f32 == o.f32;
+           f32 == o.f32 && cols == o.cols;
   }
 };
 constexpr int kMapCache = 16;
@@ -158,15 +160,16 @@ thread_local CUtensorMap t_maps[kMapCache];
 thread_local int t_map_next = 0;
 
 mw_status make_map(CUtensorMap* m, const void* ptr, int rows, int BH, int d, const char* name,
-                   int box_rows = mw::kTileRows, bool f32 = false) {
-  const MapKey key{ptr, rows, BH, d, box_rows, f32};
+                   int box_rows = mw::kTileRows, bool f32 = false, int cols = 0) {
+  if (cols == 0) cols = d;
+  const MapKey key{ptr, rows, BH, d, box_rows, f32, cols};
   for (int i = 0; i < kMapCache; ++i) {
     if (t_map_keys[i].ptr != nullptr && t_map_keys[i] == key) {
       *m = t_maps[i];
       return MW_OK;
     }
   }
-  MW_TRY(encode_map(m, ptr, rows, BH, d, name, box_rows, f32));
+  MW_TRY(encode_map(m, ptr, rows, BH, d, name, box_rows, f32, cols));
   const int slot = t_map_next;
   t_map_next = (t_map_next + 1) % kMapCache;
   t_map_keys[slot] = key;
@@ -629,7 +632,7 @@ mw_status mw_bca_bwd_stage(int stage, const void* q, const void* k, const void* 
     MW_TRY(make_map(&tk, k, static_cast<int>(N), BH, d, "k"));
     MW_TRY(make_map(&tv, v, static_cast<int>(N), BH, d, "v"));
     MW_TRY(make_map(&tdo, dout, static_cast<int>(N), BH, d, "dout", qrows));
-    MW_TRY(make_map(&tdq, dq_acc, N_pad, BH, D, "dq_acc", 32, true));
+    MW_TRY(make_map(&tdq, dq_acc, N_pad, BH, D, "dq_acc", 32, true, d));
     CUtensorMap tbias = tdq;  // d = 128: unused
     if (bias != nullptr) MW_TRY(encode_bias_map(&tbias, bias, N_pad, BH, qrows));
     mw::BwdParams p{};

@@ -12,31 +12,37 @@
 //           dP^T = V dO^T           (tcgen05 -> TMEM; d = 64: + the -D bias)
 //           P^T  = exp2(scale log2e S^T - LSE2)     (registers)
 //           dS^T = P^T (dP^T - D)                   (registers)
-//           P^T (bf16) -> TMEM; dS^T (bf16) -> shared memory (d = 128: to
-//                 TMEM as well, beside P^T)
+//           P^T (bf16) -> TMEM; dS^T (bf16) -> shared memory
 //           dV += P^T dO            (tcgen05, A = P^T from TMEM)
-//           dK += dS^T Q            (d = 64: A from shared memory; d = 128:
-//                                    from TMEM)
+//           dK += dS^T Q            (A from shared memory)
 //           d = 64 : dQ_j = dS K    (query rows in TMEM lanes)
 //           d = 128: dQ_j^T = K^T dS^T (head-dim columns in TMEM lanes)
-//           dQacc += dQ_j  (fp32: TMA reduce-add of swizzled shared-memory
-//                           boxes at d = 64, red.global at d = 128)
+//           dQacc += dQ_j  (fp32: TMA reduce-add of swizzled shared-memory boxes)
 //   post: dQ = scale * dQacc -> bf16
 //
-// Software pipeline: the P/dS warps copy S^T and dP^T into registers and
-// release their TMEM columns at once, so S^T and dP^T of step j+1 are
-// computed while they work on step j; P^T is handed over before dS is
-// computed, so dV_j overlaps that math; dK, dQ of step j run while the P/dS
-// warps start step j+1.  At d = 128 TMEM holds one block X for S^T, then
-// dP^T, then P^T / dS^T in turn, so those steps follow one another.
+// Software pipeline: the P/dS warps copy S^T and dP^T into registers at once;
+// P^T is handed over before dS is computed, so dV_j overlaps that math; dK, dQ
+// of step j run while the P/dS warps start step j+1.  d = 64: all results
+// have TMEM columns of their own, and S^T, dP^T of step j+1 are computed as
+// soon as step j's are in registers.  d = 128: P^T overwrites S^T and dQ^T
+// overwrites dP^T, one issuer runs dP_j, dV_j, S_{j+1} and the other dQ_j,
+// dK_j: S_{j+1} and its softmax overlap dQ_j and dK_j, dS_j overlaps dV_j and
+// S_{j+1}.  (One block for S^T, dP^T and P^T / dS^T in turn, with scalar
+// reductions from registers, took 2.92 ms on 16 heads of 21 x 880 tokens, this
+// form 2.50 ms; 16 heads of 72 channels, 16 x 880: 1.40 -> 1.30 ms.  What
+// bounds it: the shared-memory data path, which the MMAs' operands, the
+// copies, dS^T and the dQ boxes keep busy nearly all the time, and the dQ
+// traffic of 64 KB a step; without the reductions the same kernel takes
+// 1.97 ms.  Boxes of 16 rows were slower, 2.66 ms, and so were reductions from
+// registers, scalar 2.91 ms or as 16-byte vectors, which slow the MMAs down.)
 //
 // Roles (512 threads): warps 0-7 P/dS (two warpgroups, one half of the query
 // columns each, one key row per thread), warps 8-11 dQ drain, warp 12 TMA
-// producer, warp 13 MMA issuer (d = 64: warp 13 issues S^T, dV, dP^T and
-// warp 14 dK, dQ).
+// producer, warps 13 and 14 MMA issuers (warp 13 S^T, dV, dP^T, warp 14 dK,
+// dQ, so that one warp's barrier waits do not leave the tensor core idle).
 // TMEM (512 columns): d = 64: dV [0,64), dK [64,128), S^T [128,256),
 // dP^T [256,384), P^T [384,448), dQ [448,512); d = 128: dV [0,128),
-// dK [128,256), X [256,384), dQ^T [384,512).
+// dK [128,256), S^T and P^T [256,384), dP^T and dQ^T [384,512).
 // CTA order: head by head, or (where the host's model of the launch says it
 // ends sooner) in head groups whose key tiles run side by side, the first
 // (longest) ones first.
@@ -60,74 +66,71 @@ struct BwdLayout {
   static constexpr int QREGION = QN * 128;           // region of a QN-row tile
   static constexpr int KTILE = REG * KREGION;
   static constexpr int QTILE = REG * QREGION;
-  static constexpr int STAGES = (D == 64) ? 3 : 2;   // Q and dO tiles in flight
+  static constexpr int QSTAGES = (D == 64) ? 3 : 2;  // Q tiles in flight
+  static constexpr int DOSTAGES = (D == 64) ? 3 : 1; // dO tiles in flight
   static constexpr int DS_BYTES = (QN / 64) * KREGION;  // dS^T: 128 key rows x QN columns
   // d = 64: two dS^T buffers, so dS^T_{j+1} is written while dK_j / dQ_j read dS^T_j
   static constexpr int DS_BUFS = (D == 64) ? 2 : 1;
-  // d = 64: per drain warp, one 32 x 32 f32 box with the 128-byte swizzle (the
-  // TMA reduce-add source); 1024-byte aligned
-  static constexpr int STG_BYTES = DQT ? 0 : 4 * 32 * 32 * 4;
+  // per drain warp, one (d = 128: two) 32 x 32 f32 boxes with the 128-byte
+  // swizzle (the TMA reduce-add source); 1024-byte aligned
+  static constexpr int BOX_BYTES = 32 * 32 * 4;
+  static constexpr int STG_BYTES = (DQT ? 2 : 1) * 4 * BOX_BYTES;
   // d = 64: the per-query LSE and D terms enter S^T and dP^T through one
   // tf32 MMA each (a QN x 32-byte bias tile in each Q stage, all-ones A
   // rows), so the P/dS warps read no LSE or D rows from shared memory
   static constexpr bool FOLD = (D == 64);
   static constexpr int BIAS_BYTES = FOLD ? QN * 32 : 0;
   static constexpr int QSTRIDE = QTILE + BIAS_BYTES;  // one Q stage
+  // d = 128: LSE rows come with the Q stages, D rows with dO in two buffers
+  // (step j-2's is free: dO_j is loaded after dV_{j-1}, and so after dS_{j-2})
   static constexpr int VEC_BYTES = FOLD ? 0 : QN * 4;
   static constexpr int ONES_BYTES = FOLD ? 512 : 0;   // two 256-byte atoms of A rows
   static constexpr int OFF_K = 0;
   static constexpr int OFF_V = OFF_K + KTILE;
   static constexpr int OFF_Q = OFF_V + KTILE;
-  static constexpr int OFF_DO = OFF_Q + STAGES * QSTRIDE;
-  static constexpr int OFF_DS = OFF_DO + STAGES * QTILE;
+  static constexpr int OFF_DO = OFF_Q + QSTAGES * QSTRIDE;
+  static constexpr int OFF_DS = OFF_DO + DOSTAGES * QTILE;
   static constexpr int OFF_STG = OFF_DS + DS_BUFS * DS_BYTES;
   static constexpr int OFF_LSE = OFF_STG + STG_BYTES;
-  static constexpr int OFF_DELTA = OFF_LSE + STAGES * VEC_BYTES;
-  static constexpr int OFF_ONES = OFF_DELTA + STAGES * VEC_BYTES;
+  static constexpr int OFF_DELTA = OFF_LSE + QSTAGES * VEC_BYTES;
+  static constexpr int OFF_ONES = OFF_DELTA + 2 * VEC_BYTES;
   static constexpr int OFF_BAR = OFF_ONES + ONES_BYTES;
-  // kv_full, q_full[S], q_empty[S], do_full[S], do_empty[S], s_full, s_free,
-  // dp_full, dp_free, pt_ready, pt_free, p_ready, dq_full, dq_free,
+  // kv_full, q_full, q_empty [QSTAGES], do_full, do_empty [DOSTAGES], s_full,
+  // s_free, dp_full, dp_free, pt_ready, pt_free, p_ready, dq_full, dq_free,
   // ds_free[DS_BUFS], dkv_full
-  static constexpr int NBAR = 1 + 4 * STAGES + 10 + DS_BUFS;
+  static constexpr int NBAR = 1 + 2 * (QSTAGES + DOSTAGES) + 10 + DS_BUFS;
   static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
   static constexpr int BYTES = OFF_MISC + 16;
-  // d = 128 has no room for separate S^T / dP^T / P^T-dS^T columns: one
-  // 128-column block X holds them in turn (each is copied to registers
-  // before the next one lands there)
-  static constexpr bool SHARED_X = (D == 128);
-  static constexpr bool TWO_ISSUERS = !SHARED_X;  // MMA issue split over warps 13 and 14
+  // d = 128 has no room for separate S^T, dP^T, P^T and dQ^T columns: P^T
+  // overwrites S^T and dQ^T overwrites dP^T (each is in registers by then)
+  static constexpr bool PAIRED = (D == 128);
   static constexpr uint32_t DV_COL = 0;
   static constexpr uint32_t DK_COL = D;
   static constexpr uint32_t S_COL = 2 * D;
-  static constexpr uint32_t DP_COL = SHARED_X ? S_COL : 2 * D + QN;
-  // P^T (bf16 pairs; at d = 128 followed by dS^T).  At d = 64 dK reads dS^T
-  // from shared memory (the copy dQ reads too), so dQ has columns of its own.
-  static constexpr uint32_t PDS_COL = SHARED_X ? S_COL : 384u;
-  static constexpr uint32_t DQ_COL = SHARED_X ? 384u : 448u;
+  static constexpr uint32_t DP_COL = 2 * D + QN;
+  static constexpr uint32_t P_COL = PAIRED ? S_COL : 384u;  // P^T, bf16 pairs
+  static constexpr uint32_t DQ_COL = PAIRED ? DP_COL : 448u;
   static constexpr int THREADS = 512;
   // CTA order in head groups (BwdParams::head_groups).  The 128-wide MMA
   // variant runs head by head with the key tile taken straight from the CTA
   // index: with the group decode it measured 2-3% slower even in head-by-
   // head order, and its training shapes have no tail for groups to win back.
   static constexpr bool GROUPED = !(D == 128 && DM == 128);
-  // registers per thread after the re-split: the P/dS warpgroups get more,
-  // the drain warpgroup and the control warpgroup (TMA, MMA) less; the three
-  // shares add up to exactly the launch's 512 threads x 128 registers (at
-  // d = 64, 168 / 88 / 88 measured 1.4% faster than 176 / 80 / 80 and
-  // compiles without spills)
+  // registers per thread after the re-split between the P/dS warpgroups, the
+  // drain and the control warpgroup (TMA, MMA); the three shares add up to
+  // exactly the launch's 512 threads x 128 registers (at d = 64, 168 / 88 / 88
+  // measured 1.4% faster than 176 / 80 / 80 and compiles without spills; at
+  // d = 128 the drain holds all 128 columns of dQ^T, so that their TMEM can
+  // take the next dP^T before they are staged)
   static constexpr int REGS_LAUNCH = 128;
-  static constexpr int REGS_PDS = (D == 64) ? 168 : 152;
-  static constexpr int REGS_DRAIN = (D == 64) ? 88 : 104;
-  static constexpr int REGS_CONTROL = (D == 64) ? 88 : 104;
+  static constexpr int REGS_PDS = (D == 64) ? 168 : 144;
+  static constexpr int REGS_DRAIN = (D == 64) ? 88 : 144;
+  static constexpr int REGS_CONTROL = (D == 64) ? 88 : 80;
   static_assert(256 * REGS_PDS + 128 * REGS_DRAIN + 128 * REGS_CONTROL == THREADS * REGS_LAUNCH,
                 "register re-split must hand out exactly the launch's registers");
-  static_assert(SHARED_X ? (2 * D + QN <= 384) : (2 * D + 2 * QN <= 384), "TMEM columns");
+  static_assert(2 * D + 2 * QN <= (PAIRED ? 512 : 384), "TMEM columns");
   static_assert(BYTES <= 232448, "shared memory");
 };
-
-__device__ __forceinline__ void red_add(float* addr, float a) {
-  asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(a) : "memory");
-}
 
 template <int D, int DM>
 __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
@@ -136,7 +139,8 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
                    const __grid_constant__ CUtensorMap tm_dq,
                    const __grid_constant__ CUtensorMap tm_bias, const BwdParams p) {
   using L = BwdLayout<D, DM>;
-  constexpr int NS = L::STAGES;
+  constexpr int NQ = L::QSTAGES;
+  constexpr int ND = L::DOSTAGES;
   constexpr int QN = L::QN;
   constexpr int CW = L::CW;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -186,10 +190,10 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
   uint64_t* kv_full = bars;
   uint64_t* q_full = bars + 1;
-  uint64_t* q_empty = q_full + NS;
-  uint64_t* do_full = q_empty + NS;
-  uint64_t* do_empty = do_full + NS;
-  uint64_t* s_full = do_empty + NS;
+  uint64_t* q_empty = q_full + NQ;
+  uint64_t* do_full = q_empty + NQ;
+  uint64_t* do_empty = do_full + ND;
+  uint64_t* s_full = do_empty + ND;
   uint64_t* s_free = s_full + 1;
   uint64_t* dp_full = s_free + 1;
   uint64_t* dp_free = dp_full + 1;
@@ -247,9 +251,11 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
     *head_slot = bh_decoded;
     *tile_slot = kt;
     mbar_init(kv_full, 1);
-    for (int s = 0; s < NS; ++s) {
+    for (int s = 0; s < NQ; ++s) {
       mbar_init(&q_full[s], 1);
       mbar_init(&q_empty[s], 1);
+    }
+    for (int s = 0; s < ND; ++s) {
       mbar_init(&do_full[s], 1);
       mbar_init(&do_empty[s], 1);
     }
@@ -263,7 +269,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
     mbar_init(dq_full, 1);
     mbar_init(dq_free, 4);
     for (int b = 0; b < L::DS_BUFS; ++b) mbar_init(&ds_free[b], 1);
-    mbar_init(dkv_full, L::TWO_ISSUERS ? 2 : 1);
+    mbar_init(dkv_full, 2);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -302,46 +308,46 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       }
       int issued_q = 0, issued_do = 0;
       for (int j = 0; j < n_q; ++j) {
-        const int st = j % NS;
-        const uint32_t ph = (j / NS) & 1;
+        const int st = j % NQ;
         const int q0 = (m_begin + (j + q_rot) % n_q) * QN;
         const size_t voff = static_cast<size_t>(bh) * p.N_pad + q0;
-        if (!mbar_wait(&q_empty[st], ph ^ 1, ctl)) break;
+        if (!mbar_wait(&q_empty[st], ((j / NQ) & 1) ^ 1, ctl)) break;
         if (!p.debug_skip_q) {
           mbar_arrive_expect_tx(&q_full[st], L::QTILE + L::BIAS_BYTES + L::VEC_BYTES);
           for (int r = 0; r < L::REG; ++r)
             tma_load_3d(sQ + st * L::QSTRIDE + r * L::QREGION, &tm_q, &q_full[st], 64 * r, q0, bh);
-          if constexpr (L::FOLD)
+          if constexpr (L::FOLD) {
             tma_load_3d(sQ + st * L::QSTRIDE + L::QTILE, &tm_bias, &q_full[st], 0, q0, bh);
-          else
+          } else {
             bulk_load(sLSE + st * QN, p.lse2 + voff, L::VEC_BYTES, &q_full[st]);
+          }
           ++issued_q;
         }
-        if (!mbar_wait(&do_empty[st], ph ^ 1, ctl)) break;
-        mbar_arrive_expect_tx(&do_full[st], L::QTILE + L::VEC_BYTES);
+        const int sd = j % ND;
+        if (!mbar_wait(&do_empty[sd], ((j / ND) & 1) ^ 1, ctl)) break;
+        mbar_arrive_expect_tx(&do_full[sd], L::QTILE + L::VEC_BYTES);
         for (int r = 0; r < L::REG; ++r)
-          tma_load_3d(sDO + st * L::QTILE + r * L::QREGION, &tm_do, &do_full[st], 64 * r, q0, bh);
-        if constexpr (!L::FOLD) bulk_load(sDelta + st * QN, p.delta + voff, L::VEC_BYTES, &do_full[st]);
+          tma_load_3d(sDO + sd * L::QTILE + r * L::QREGION, &tm_do, &do_full[sd], 64 * r, q0, bh);
+        if constexpr (!L::FOLD)
+          bulk_load(sDelta + (j & 1) * QN, p.delta + voff, L::VEC_BYTES, &do_full[sd]);
         ++issued_do;
       }
       if (*abort_flag) {
         drain_wait(kv_full, 0, p.budget_ns);
-        for (int j = max(0, issued_q - NS); j < issued_q; ++j)
-          drain_wait(&q_full[j % NS], (j / NS) & 1, p.budget_ns);
-        for (int j = max(0, issued_do - NS); j < issued_do; ++j)
-          drain_wait(&do_full[j % NS], (j / NS) & 1, p.budget_ns);
+        for (int j = max(0, issued_q - NQ); j < issued_q; ++j)
+          drain_wait(&q_full[j % NQ], (j / NQ) & 1, p.budget_ns);
+        for (int j = max(0, issued_do - ND); j < issued_do; ++j)
+          drain_wait(&do_full[j % ND], (j / ND) & 1, p.budget_ns);
       }
     }
-  } else if (warp == 13 || (L::TWO_ISSUERS && warp == 14)) {
+  } else if (warp == 13 || warp == 14) {
     // ------------------------------------------------------------ MMA issuers (whole warps)
     const int n_q = sweep().n_q;
-    // d = 64: warp 13 issues S^T, dV and dP^T, warp 14 dK and dQ, so that one
-    // warp's waits never leave the tensor core's short queue empty.  They
-    // share no TMEM columns; the P/dS barriers order their operands.
-    // d = 128 (S^T, dP^T, P^T and dS^T share columns): warp 13 issues all.
+    // warp 13 issues S^T, dV and dP^T, warp 14 dK and dQ, so that one warp's
+    // waits never leave the tensor core's short queue empty; the P/dS and
+    // drain barriers order what shares operands or TMEM columns
     {
-      const bool role_a = !L::TWO_ISSUERS || warp == 13;  // S^T, dV, dP^T
-      const bool role_b = !L::TWO_ISSUERS || warp == 14;  // dK, dQ
+      const bool role_a = warp == 13;  // S^T, dV, dP^T
       constexpr uint32_t idesc_s = idesc_bf16_f32(128, QN, false, false);    // S^T, dP^T
       constexpr uint32_t idesc_tn = idesc_bf16_f32(128, DM, false, true);    // dV, dK
       // d = 64: dQ = dS K (M = query rows); d = 128: dQ^T = K^T dS^T (M = head dim)
@@ -376,129 +382,140 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
           umma_ss(tmem + d_col, sdesc_add(a, ka), sdesc_add(b, kq), idesc_s, kk > 0 ? 1u : 0u);
         }
       };
-      // TMEM columns of the k-th 16-query slice of P^T and of dS^T (bf16 pairs)
+      // TMEM column of the k-th 16-query slice of P^T (bf16 pairs; at d = 128
+      // each warpgroup's half lies in its own 64 columns of S^T)
       auto pt_col = [](int kk) -> uint32_t {
-        return L::SHARED_X ? L::PDS_COL + (kk >> 2) * 64 + (kk & 3) * 8 : L::PDS_COL + kk * 8;
+        return L::PAIRED ? L::P_COL + (kk >> 2) * 64 + (kk & 3) * 8 : L::P_COL + kk * 8;
       };
-      auto dst_col = [](int kk) -> uint32_t {
-        return L::SHARED_X ? L::PDS_COL + (kk >> 2) * 64 + 32 + (kk & 3) * 8
-                           : L::PDS_COL + QN / 2 + kk * 8;
+      auto issue_dv = [&](int j) {  // dV += P^T dO_j
+        const uint32_t do_mn = sdesc_add(do_mn0, (j % ND) * L::QTILE);
+#pragma unroll
+        for (int kk = 0; kk < QN / 16; ++kk)
+          umma_ts(tmem + L::DV_COL, tmem + pt_col(kk), sdesc_add(do_mn, kk * 2048), idesc_tn,
+                  (j > 0 || kk > 0) ? 1u : 0u);
+      };
+      auto issue_dk = [&](int j) {  // dK += dS^T Q_j, dS^T read from shared memory (K-major)
+        const uint32_t ds_kmaj = sdesc_add(ds_kmaj0, (j % L::DS_BUFS) * L::DS_BYTES);
+        const uint32_t q_mn = sdesc_add(q_mn0, (j % NQ) * L::QSTRIDE);
+#pragma unroll
+        for (int kk = 0; kk < QN / 16; ++kk)
+          umma_ss(tmem + L::DK_COL, sdesc_add(ds_kmaj, (kk >> 2) * L::KREGION + (kk & 3) * 32),
+                  sdesc_add(q_mn, kk * 2048), idesc_tn, (j > 0 || kk > 0) ? 1u : 0u);
+      };
+      auto issue_dq = [&](int j) {
+        const uint32_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
+#pragma unroll
+        for (int kk = 0; kk < kTileRows / 16; ++kk) {
+          if constexpr (L::DQT)   // A = K^T (MN-major over d), B = dS^T (MN-major over queries)
+            umma_ss(tmem + L::DQ_COL, sdesc_add(k_mn, kk * 2048), sdesc_add(ds_mn, kk * 2048),
+                    idesc_dq, kk > 0 ? 1u : 0u);
+          else                    // A = dS (MN-major over queries), B = K (MN-major over d)
+            umma_ss(tmem + L::DQ_COL, sdesc_add(ds_mn, kk * 2048), sdesc_add(k_mn, kk * 2048),
+                    idesc_dq, kk > 0 ? 1u : 0u);
+        }
       };
       bool ok = warp_wait(kv_full, 0, ctl);
-      if (ok && role_a) ok = warp_wait(&q_full[0], 0, ctl);
-      tc_fence_after();
-      if (ok && role_a) {
-        issue_kmajor(L::S_COL, k_kmaj, q_kmaj0);
-        add_bias(L::S_COL, ones_l, 0);
-        umma_commit(s_full);
-        if (L::SHARED_X) ok = warp_wait(s_free, 0, ctl);  // X holds S^T_0 until read
-        if (ok) ok = warp_wait(&do_full[0], 0, ctl);
-        tc_fence_after();
-      }
-      if (ok && role_a) {
-        issue_kmajor(L::DP_COL, v_kmaj, do_kmaj0);
-        add_bias(L::DP_COL, ones_d, 0);
-        umma_commit(dp_full);
-      }
-      for (int j = 0; ok && j < n_q; ++j) {
-        const int st = j % NS;
-        const int st1 = (j + 1) % NS;
-        const uint32_t ph1 = ((j + 1) / NS) & 1;
-        const bool more = j + 1 < n_q;
-        const uint32_t do_mn = sdesc_add(do_mn0, st * L::QTILE);
-        const uint32_t q_mn = sdesc_add(q_mn0, st * L::QSTRIDE);
+      if constexpr (L::PAIRED) {
         if (role_a) {
-          if (!L::SHARED_X && more) {
-            // S^T of the next step as soon as the P/dS warps hold S^T_j
-            if (!(ok = warp_wait(s_free, j & 1, ctl))) break;
-            if (!(ok = warp_wait(&q_full[st1], ph1, ctl))) break;
+          // dP_j, dV_j, S_{j+1}: MMAs of one issuer run in order, so S_{j+1}
+          // may land on P_j once dV_j is issued
+          if (ok) ok = warp_wait(&q_full[0], 0, ctl);
+          if (ok) {
             tc_fence_after();
-            issue_kmajor(L::S_COL, k_kmaj, sdesc_add(q_kmaj0, st1 * L::QSTRIDE));
-            add_bias(L::S_COL, ones_l, st1);
+            issue_kmajor(L::S_COL, k_kmaj, q_kmaj0);
             umma_commit(s_full);
           }
-          // dV += P^T dO_j as soon as P^T_j is in TMEM (while dS_j is computed)
-          if (!(ok = warp_wait(pt_ready, j & 1, ctl))) break;
-          tc_fence_after();
-#pragma unroll
-          for (int kk = 0; kk < QN / 16; ++kk)
-            umma_ts(tmem + L::DV_COL, tmem + pt_col(kk), sdesc_add(do_mn, kk * 2048),
-                    idesc_tn, (j > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(&do_empty[st]);
-          if (!L::SHARED_X) umma_commit(pt_free);
-          if (!L::SHARED_X && more) {
-            // dP^T of the next step once the P/dS warps hold dP^T_j
-            if (!(ok = warp_wait(dp_free, j & 1, ctl))) break;
-            if (!(ok = warp_wait(&do_full[st1], ph1, ctl))) break;
+          for (int j = 0; ok && j < n_q; ++j) {
+            if (!(ok = warp_wait(&do_full[j % ND], (j / ND) & 1, ctl))) break;
+            // dQ_{j-1} is in the drain's registers: its columns take dP_j
+            if (j > 0 && !(ok = warp_wait(dq_free, (j - 1) & 1, ctl))) break;
             tc_fence_after();
-            issue_kmajor(L::DP_COL, v_kmaj, sdesc_add(do_kmaj0, st1 * L::QTILE));
-            add_bias(L::DP_COL, ones_d, st1);
+            issue_kmajor(L::DP_COL, v_kmaj, sdesc_add(do_kmaj0, (j % ND) * L::QTILE));
             umma_commit(dp_full);
+            if (!(ok = warp_wait(pt_ready, j & 1, ctl))) break;
+            tc_fence_after();
+            issue_dv(j);
+            umma_commit(&do_empty[j % ND]);
+            if (j + 1 < n_q) {
+              const int st1 = (j + 1) % NQ;
+              if (!(ok = warp_wait(&q_full[st1], ((j + 1) / NQ) & 1, ctl))) break;
+              tc_fence_after();
+              issue_kmajor(L::S_COL, k_kmaj, sdesc_add(q_kmaj0, st1 * L::QSTRIDE));
+              umma_commit(s_full);
+            }
+          }
+        } else {
+          for (int j = 0; ok && j < n_q; ++j) {
+            // dS_j is in shared memory (and so dP_j in registers)
+            if (!(ok = warp_wait(p_ready, j & 1, ctl))) break;
+            tc_fence_after();
+            issue_dq(j);
+            umma_commit(dq_full);
+            issue_dk(j);
+            umma_commit(&q_empty[j % NQ]);
+            umma_commit(&ds_free[j % L::DS_BUFS]);
           }
         }
-        if (role_b) {
-          if (!(ok = warp_wait(p_ready, j & 1, ctl))) break;
+      } else {
+        if (ok && role_a) ok = warp_wait(&q_full[0], 0, ctl);
+        tc_fence_after();
+        if (ok && role_a) {
+          issue_kmajor(L::S_COL, k_kmaj, q_kmaj0);
+          add_bias(L::S_COL, ones_l, 0);
+          umma_commit(s_full);
+          ok = warp_wait(&do_full[0], 0, ctl);
           tc_fence_after();
-          if constexpr (!L::SHARED_X) {
-            // d = 64: dQ_j first, so the drain starts while dK_j runs
+        }
+        if (ok && role_a) {
+          issue_kmajor(L::DP_COL, v_kmaj, do_kmaj0);
+          add_bias(L::DP_COL, ones_d, 0);
+          umma_commit(dp_full);
+        }
+        for (int j = 0; ok && j < n_q; ++j) {
+          const int st1 = (j + 1) % NQ;
+          const uint32_t ph1 = ((j + 1) / NQ) & 1;
+          const bool more = j + 1 < n_q;
+          static_assert(L::PAIRED || NQ == ND, "stage indices are shared");
+          if (role_a) {
+            if (more) {
+              // S^T of the next step as soon as the P/dS warps hold S^T_j
+              if (!(ok = warp_wait(s_free, j & 1, ctl))) break;
+              if (!(ok = warp_wait(&q_full[st1], ph1, ctl))) break;
+              tc_fence_after();
+              issue_kmajor(L::S_COL, k_kmaj, sdesc_add(q_kmaj0, st1 * L::QSTRIDE));
+              add_bias(L::S_COL, ones_l, st1);
+              umma_commit(s_full);
+            }
+            // dV += P^T dO_j as soon as P^T_j is in TMEM (while dS_j is computed)
+            if (!(ok = warp_wait(pt_ready, j & 1, ctl))) break;
+            tc_fence_after();
+            issue_dv(j);
+            umma_commit(&do_empty[j % ND]);
+            umma_commit(pt_free);
+            if (more) {
+              // dP^T of the next step once the P/dS warps hold dP^T_j
+              if (!(ok = warp_wait(dp_free, j & 1, ctl))) break;
+              if (!(ok = warp_wait(&do_full[st1], ph1, ctl))) break;
+              tc_fence_after();
+              issue_kmajor(L::DP_COL, v_kmaj, sdesc_add(do_kmaj0, st1 * L::QTILE));
+              add_bias(L::DP_COL, ones_d, st1);
+              umma_commit(dp_full);
+            }
+          }
+          if (!role_a) {
+            if (!(ok = warp_wait(p_ready, j & 1, ctl))) break;
+            tc_fence_after();
+            // dQ_j first, so the drain starts while dK_j runs
             if (j > 0) {
               if (!(ok = warp_wait(dq_free, (j - 1) & 1, ctl))) break;
               tc_fence_after();
             }
-            const uint32_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
-#pragma unroll
-            for (int kk = 0; kk < kTileRows / 16; ++kk)
-              umma_ss(tmem + L::DQ_COL, sdesc_add(ds_mn, kk * 2048), sdesc_add(k_mn, kk * 2048),
-                      idesc_dq, kk > 0 ? 1u : 0u);
+            issue_dq(j);
             umma_commit(dq_full);
+            issue_dk(j);
+            umma_commit(&q_empty[j % NQ]);
+            umma_commit(&ds_free[j % L::DS_BUFS]);
           }
-          // dK += dS^T Q_j (d = 64: dS^T read from shared memory, K-major)
-          const uint32_t ds_kmaj = sdesc_add(ds_kmaj0, (j % L::DS_BUFS) * L::DS_BYTES);
-#pragma unroll
-          for (int kk = 0; kk < QN / 16; ++kk) {
-            if constexpr (L::SHARED_X)
-              umma_ts(tmem + L::DK_COL, tmem + dst_col(kk), sdesc_add(q_mn, kk * 2048),
-                      idesc_tn, (j > 0 || kk > 0) ? 1u : 0u);
-            else
-              umma_ss(tmem + L::DK_COL, sdesc_add(ds_kmaj, (kk >> 2) * L::KREGION + (kk & 3) * 32),
-                      sdesc_add(q_mn, kk * 2048), idesc_tn, (j > 0 || kk > 0) ? 1u : 0u);
-          }
-          umma_commit(&q_empty[st]);
-          if constexpr (!L::SHARED_X) umma_commit(&ds_free[j % L::DS_BUFS]);
-        }
-        if (L::SHARED_X && more) {
-          // X is free once dV/dK have read P^T/dS^T (issue order): S^T of the
-          // next step, then its dP^T once the P/dS warps have read that S^T
-          if (!(ok = warp_wait(&q_full[st1], ph1, ctl))) break;
-          tc_fence_after();
-          issue_kmajor(L::S_COL, k_kmaj, sdesc_add(q_kmaj0, st1 * L::QSTRIDE));
-            add_bias(L::S_COL, ones_l, st1);
-          umma_commit(s_full);
-          if (!(ok = warp_wait(s_free, (j + 1) & 1, ctl))) break;
-          if (!(ok = warp_wait(&do_full[st1], ph1, ctl))) break;
-          tc_fence_after();
-          issue_kmajor(L::DP_COL, v_kmaj, sdesc_add(do_kmaj0, st1 * L::QTILE));
-            add_bias(L::DP_COL, ones_d, st1);
-          umma_commit(dp_full);
-        }
-        if (L::SHARED_X && role_b) {
-          // dQ of this step, once the drain has read the previous one
-          if (j > 0) {
-            if (!(ok = warp_wait(dq_free, (j - 1) & 1, ctl))) break;
-            tc_fence_after();
-          }
-          const uint32_t ds_mn = sdesc_add(ds_mn0, (j % L::DS_BUFS) * L::DS_BYTES);
-#pragma unroll
-          for (int kk = 0; kk < kTileRows / 16; ++kk) {
-            if constexpr (L::DQT)   // A = K^T (MN-major over d), B = dS^T (MN-major over queries)
-              umma_ss(tmem + L::DQ_COL, sdesc_add(k_mn, kk * 2048), sdesc_add(ds_mn, kk * 2048),
-                      idesc_dq, kk > 0 ? 1u : 0u);
-            else                    // A = dS (MN-major over queries), B = K (MN-major over d)
-              umma_ss(tmem + L::DQ_COL, sdesc_add(ds_mn, kk * 2048), sdesc_add(k_mn, kk * 2048),
-                      idesc_dq, kk > 0 ? 1u : 0u);
-          }
-          umma_commit(dq_full);
-          umma_commit(&ds_free[j % L::DS_BUFS]);
         }
       }
       if (ok) umma_commit(dkv_full);  // one arrival per issuing warp
@@ -517,10 +534,9 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(wq * 32) << 16);
     const uint32_t s_addr = lane_base + L::S_COL + CW * wg;
     const uint32_t dp_addr = lane_base + L::DP_COL + CW * wg;
-    // P^T / dS^T destinations: within this warpgroup's own 64 X columns
-    // (d = 128), or in the separate P^T and dS^T blocks (d = 64)
-    const uint32_t pds_p = lane_base + (L::SHARED_X ? L::PDS_COL + 64 * wg : L::PDS_COL + 32 * wg);
-    const uint32_t pds_s = L::SHARED_X ? pds_p + 32 : pds_p + QN / 2;
+    // P^T: over this warpgroup's own 64 columns of S^T (d = 128), or in
+    // columns of its own (d = 64)
+    const uint32_t p_addr = lane_base + L::P_COL + (L::PAIRED ? 64 : 32) * wg;
     const float sl2 = p.scale_log2;
     // this thread's dS^T row segment: region (CW wg) / 64, chunks from (CW wg % 64) / 8
     const int c0 = CW * wg;
@@ -529,10 +545,10 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
     const int sw = j_local & 7;
     bool ok = true;
     for (int j = 0; j < n_q; ++j) {
-      const int st = j % NS;
+      const int st = j % NQ;
       const int q0 = (m_begin + (j + q_rot) % n_q) * QN;
       const float* lse2 = sLSE + st * QN + c0;
-      const float* delta = sDelta + st * QN + c0;
+      const float* delta = sDelta + (j & 1) * QN + c0;
       if (!(ok = warp_wait(s_full, j & 1, ctl))) break;
       tc_fence_after();
       // d = 128: the step's LSE row (16 bytes per load), read once S^T is in
@@ -557,9 +573,11 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
 #pragma unroll
           for (int k = 0; k < 32; ++k) pr[32 * h + k] = __uint_as_float(r[h][k]);
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(s_free);
+      if constexpr (!L::PAIRED) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(s_free);
+      }
       const int lim = q_start - q0 - c0;  // columns c < lim are masked
       if constexpr (!L::FOLD) load_lse();
       const float2 sl2x2 = make_float2(sl2, sl2);
@@ -576,37 +594,33 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         for (int c = 0; c < CW; ++c)
           if (c < lim) pr[c] = 0.f;
       }
-      uint32_t dk[CW / 2];
-      uint32_t pk[L::SHARED_X ? CW / 2 : 1];  // d = 128: P^T packed alongside dS^T
-      // d = 64: P^T (bf16 pairs) -> TMEM right away, so that dV_j starts
-      // while dS_j is computed.  (d = 128: X still holds dP^T_j; P^T is stored
-      // with dS^T at the end of the step, which measured faster there.)
-      auto store_pt = [&]() {
-        uint32_t pe[CW / 2];
-#pragma unroll
-        for (int c = 0; c < CW / 2; ++c) pe[c] = pack_bf16x2(pr[2 * c], pr[2 * c + 1]);
-        tmem_st32(pds_p, pe);
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(pt_ready);
-      };
-      if constexpr (!L::SHARED_X) {
+      // P^T (bf16 pairs) -> TMEM right away, so that dV_j starts while dS_j is
+      // computed
+      if constexpr (!L::PAIRED) {
         if (j > 0) {  // dV_{j-1} has read P^T_{j-1}
           if (!(ok = warp_wait(pt_free, (j - 1) & 1, ctl))) break;
           tc_fence_after();
         }
-        store_pt();
+      }
+      {
+        uint32_t pe[CW / 2];
+#pragma unroll
+        for (int c = 0; c < CW / 2; ++c) pe[c] = pack_bf16x2(pr[2 * c], pr[2 * c + 1]);
+        tmem_st32(p_addr, pe);
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(pt_ready);
       }
       if (!(ok = warp_wait(dp_full, j & 1, ctl))) break;
       tc_fence_after();
-      // d = 128: the step's D row came with dO, which dP^T_j has read
+      uint32_t dk[CW / 2];
 #pragma unroll
       for (int h = 0; h < CW / 32; ++h) {
         uint32_t r[32];
         tmem_ld32(dp_addr + 32 * h, r);
         tmem_wait_ld();
-        if (!L::SHARED_X && h == CW / 32 - 1) {
+        if (!L::PAIRED && h == CW / 32 - 1) {
           // dP^T is in registers: its columns can take the next step's dP^T
           tc_fence_before();
           __syncwarp();
@@ -627,10 +641,6 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
           const float2 s1 = mul2(make_float2(pr[c + 2], pr[c + 3]), t1);
           dk[16 * h + 2 * k] = pack_bf16x2(s0.x, s0.y);
           dk[16 * h + 2 * k + 1] = pack_bf16x2(s1.x, s1.y);
-          if constexpr (L::SHARED_X) {
-            pk[16 * h + 2 * k] = pack_bf16x2(pr[c], pr[c + 1]);
-            pk[16 * h + 2 * k + 1] = pack_bf16x2(pr[c + 2], pr[c + 3]);
-          }
         }
       }
       // dS^T row segment -> shared memory (swizzled like a TMA 128-byte tile)
@@ -643,19 +653,10 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       for (int q = 0; q < CW / 8; ++q)
         *reinterpret_cast<uint4*>(ds_row + (((chunk0 + q) ^ sw) << 4)) =
             make_uint4(dk[4 * q], dk[4 * q + 1], dk[4 * q + 2], dk[4 * q + 3]);
-      // d = 128: P^T and dS^T -> TMEM (the dK and dV A operands)
-      if constexpr (L::SHARED_X) {
-        tmem_st32(pds_p, pk);
-        tmem_st32(pds_s, dk);
-      }
       fence_proxy_async_smem();
-      if constexpr (L::SHARED_X) tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        if (L::SHARED_X) mbar_arrive(pt_ready);
-        mbar_arrive(p_ready);
-      }
+      if (lane == 0) mbar_arrive(p_ready);
     }
     // ---- epilogue: warpgroup 0 writes dK (x scale), warpgroup 1 writes dV
     // (zeros if a wait gave up: the rows get a defined value either way)
@@ -692,7 +693,10 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       }
     }
   } else {
-    regs_dec<L::REGS_DRAIN>();
+    if constexpr (L::REGS_DRAIN > L::REGS_LAUNCH)
+      regs_inc<L::REGS_DRAIN>();
+    else
+      regs_dec<L::REGS_DRAIN>();
     // ------------------------------------------------------------ dQ drain
     const int wq = warp & 3;
     const int bh = head();
@@ -703,27 +707,33 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       if (!warp_wait(dq_full, j & 1, ctl)) break;
       tc_fence_after();
       if constexpr (L::DQT) {
-        // lanes = head-dim columns, TMEM columns = the QN query rows; one warp
-        // instruction reduces 32 consecutive head-dim columns of one row
-        float* dst = p.dq_acc + (static_cast<size_t>(bh) * p.N_pad + q0) * D + wq * 32 + lane;
-        // head-dim columns past the caller's hold zeros: no reductions for them
-        const bool col_ok = wq * 32 + lane < p.d_io;
+        // lanes = head-dim columns, TMEM columns = the QN query rows: the
+        // warp's 32 columns x QN queries leave as boxes of 32 queries (rows of
+        // 128 bytes, 16-byte chunk c of row r at c ^ (r mod 8): each store
+        // instruction fills one row, conflict-free), two in turn.  The map
+        // clips head-dim columns past the caller's; warps with none skip.
+        uint32_t r[QN / 32][32];
 #pragma unroll
-        for (int half = 0; half < QN / 64; ++half) {
-          uint32_t r0[32], r1[32];
-          tmem_ld32(lane_base + L::DQ_COL + 64 * half, r0);
-          tmem_ld32(lane_base + L::DQ_COL + 64 * half + 32, r1);
-          tmem_wait_ld();
-          if (half == QN / 64 - 1) {
-            tc_fence_before();
+        for (int c = 0; c < QN / 32; ++c) tmem_ld32(lane_base + L::DQ_COL + 32 * c, r[c]);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(dq_free);  // dQ_j is in registers
+        if (32 * wq < p.d_io) {
+#pragma unroll
+          for (int c = 0; c < QN / 32; ++c) {
+            uint8_t* stg = smem + L::OFF_STG + (2 * wq + (c & 1)) * L::BOX_BYTES;
+            if (lane == 0) bulk_wait_read<1>();  // the TMA unit has read this box
             __syncwarp();
-            if (lane == 0) mbar_arrive(dq_free);
-          }
-          if (col_ok) {
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              red_add(dst + static_cast<size_t>(64 * half + c) * D, __uint_as_float(r0[c]));
-              red_add(dst + static_cast<size_t>(64 * half + c + 32) * D, __uint_as_float(r1[c]));
+            for (int k = 0; k < 32; ++k)
+              *reinterpret_cast<uint32_t*>(stg + k * 128 + (((lane >> 2) ^ (k & 7)) << 4) +
+                                           (lane & 3) * 4) = r[c][k];
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+              tma_reduce_add_3d(&tm_dq, stg, 32 * wq, q0 + 32 * c, bh);
+              bulk_commit_group();
             }
           }
         }
@@ -733,7 +743,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         // at c ^ (r mod 8): conflict-free), and one lane hands each box to the
         // TMA unit as a reduce-add into dQacc
         static_assert(D == 64, "the drain below covers two 32-column boxes");
-        uint8_t* stg = smem + L::OFF_STG + wq * 4096;
+        uint8_t* stg = smem + L::OFF_STG + wq * L::BOX_BYTES;
         uint32_t r[2][32];
         tmem_ld32(lane_base + L::DQ_COL, r[0]);
         tmem_ld32(lane_base + L::DQ_COL + 32, r[1]);
@@ -743,7 +753,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         if (lane == 0) mbar_arrive(dq_free);  // dQ_j is in registers
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          if (lane == 0) bulk_wait_read_all();  // the box buffer was read by the TMA unit
+          if (lane == 0) bulk_wait_read<0>();  // the box buffer was read by the TMA unit
           __syncwarp();
 #pragma unroll
           for (int i = 0; i < 8; ++i)
@@ -759,11 +769,8 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       }
     }
     // every reduce-add has completed before the CTA's shared memory goes away
-    if constexpr (!L::DQT) {
-      if (lane == 0) bulk_wait_all();
-      __syncwarp();
-    }
-
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
   }
 
   __syncwarp();

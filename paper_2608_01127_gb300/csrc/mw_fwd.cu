@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
         for (int c = 0; c < (DM + 31) / 32; ++c)
           tma_store_3d(&tm_op, stage + c * kBoxBytes, 32 * c, r0 + t * kTileRows, split * p.BH + bh);
         bulk_commit_group();
-        bulk_wait_read_all();  // the boxes are read before the CTA's shared memory goes
+        bulk_wait_read<0>();  // the boxes are read before the CTA's shared memory goes
       }
     }
     if (row_valid) {

@@ -147,7 +147,7 @@ cudaError_t launch_bwd_pre(int d, int d_io, const __nv_bfloat16* o, const __nv_b
                            const float* lse, float* lse2, float* delta, float* dq_acc,
                            float* bias, float inv_scale, int BH, int N, int N_pad, cudaStream_t s);
 // tdq: f32 map over dQacc [BH, N_pad, d] with 32 x 32 boxes (128-byte
-// swizzle), the target of the d = 64 kernel's TMA reduce-adds
+// swizzle), the target of the TMA reduce-adds
 // dm: MMA width as for launch_fwd
 // tbias (d = 64): f32 map over the bias rows [BH, N_pad, 8], 8 x 128 boxes,
 // 32-byte swizzle (d = 128: any map, unused)

@@ -155,10 +155,11 @@ __device__ __forceinline__ void bulk_commit_group() {
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-// Waits until the issuing thread's committed bulk groups have finished
-// reading shared memory (the source may be overwritten afterwards).
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+// Waits until all but the issuing thread's N newest bulk groups have finished
+// reading shared memory (their sources may be overwritten afterwards).
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 
 // Waits until the issuing thread's committed bulk groups have completed.
