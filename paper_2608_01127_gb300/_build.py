@@ -3,7 +3,8 @@
 Each translation unit compiles in parallel, then one nvcc link makes the
 shared library against the shared CUDA runtime (found through an rpath to
 the toolkit; inside a PyTorch process the runtime PyTorch already loaded is
-used).  The driver is reached at run time through the runtime's entry-point
+used).  Beside it ``_lib/_mw_torch.so``, the native half of the Python binding,
+with the host compiler against PyTorch's headers.  The driver is reached at run time through the runtime's entry-point
 query, so the library loads on machines without a GPU.  A stamp of the sources' hash skips unchanged rebuilds.
 """
 from __future__ import annotations
@@ -14,6 +15,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -22,6 +24,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(PKG, "_build")
 LIB_DIR = os.path.join(PKG, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libmw_bca.so")
+TORCH_SOURCE = "mw_torch.cpp"
+TORCH_LIB_PATH = os.path.join(LIB_DIR, "_mw_torch.so")
 
 SOURCES = ["mw_abi.cu", "mw_fwd.cu", "mw_bwd.cu", "mw_commit.cu", "mw_qkv.cu"]
 HEADERS = ["mw_ptx.cuh", "mw_internal.h"]
@@ -35,6 +39,47 @@ def _nvcc() -> str:
         if cand and os.path.exists(cand):
             return cand
     raise RuntimeError("nvcc not found: the CUDA extension cannot be built")
+
+
+def _torch_module() -> list:
+    """Command that compiles the native half of the Python binding."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    lib = os.path.join(root, "lib")
+    return [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            "-I" + INCLUDE, "-isystem", os.path.join(root, "include"),
+            "-isystem", sysconfig.get_paths()["include"],
+            "-isystem", os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"),
+            os.path.join(CSRC, TORCH_SOURCE), "-o", TORCH_LIB_PATH + ".tmp",
+            "-L" + lib, "-Wl,-rpath," + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+
+
+def build_torch_module(force: bool = False) -> None:
+    """Compile _mw_torch.so if its sources, PyTorch or Python changed.  The
+    package works without it (the Python binding's own checks then run on
+    every call), so a failure is reported and the build goes on."""
+    stamp = os.path.join(BUILD_DIR, "stamp_torch")
+    try:
+        import torch
+        h = hashlib.sha256(f"{torch.__version__} {sys.version}".encode())
+        for path in (os.path.join(CSRC, TORCH_SOURCE), os.path.join(INCLUDE, "mw_bca.h")):
+            with open(path, "rb") as f:
+                h.update(f.read())
+        if not force and os.path.exists(TORCH_LIB_PATH) and os.path.exists(stamp):
+            with open(stamp) as f:
+                if f.read().strip() == h.hexdigest():
+                    return
+        r = subprocess.run(_torch_module(), capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(r.stdout + r.stderr)
+        os.replace(TORCH_LIB_PATH + ".tmp", TORCH_LIB_PATH)
+        with open(stamp, "w") as f:
+            f.write(h.hexdigest())
+    except Exception as e:  # noqa: BLE001
+        if os.path.exists(TORCH_LIB_PATH):
+            os.remove(TORCH_LIB_PATH)  # never one of other sources
+        sys.stderr.write(f"{TORCH_SOURCE}: not built, calls take the longer way: {e}\n")
 
 
 def _digest() -> str:
@@ -54,6 +99,14 @@ def build(verbose: bool = False, force: bool = False, ptxas_info: bool = False) 
     """Compile the library if its sources changed; returns the .so path."""
     os.makedirs(BUILD_DIR, exist_ok=True)
     os.makedirs(LIB_DIR, exist_ok=True)
+    with cf.ThreadPoolExecutor(max_workers=1) as ex:
+        native = ex.submit(build_torch_module, force)
+        path = _build_library(verbose, force, ptxas_info)
+        native.result()
+    return path
+
+
+def _build_library(verbose: bool, force: bool, ptxas_info: bool) -> str:
     stamp = os.path.join(BUILD_DIR, "stamp")
     digest = _digest()
     if not force and os.path.exists(LIB_PATH) and os.path.exists(stamp):
