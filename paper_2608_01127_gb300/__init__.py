@@ -67,8 +67,9 @@ _lib: Optional[ctypes.CDLL] = None
 # allocations in native code.  Calls that the host bounds, a call's wall time:
 # forward of 2 heads x 256 tokens 20.6 -> 6.8 us, streaming step against one
 # committed chunk 43.0 -> 15.9 us, forward and backward of 16 heads x 1760
-# tokens through autograd 286 -> 173 us.  Each function returns None for arguments it does not take; the checks here then
-# follow.  None until the library is loaded, or when the module was not built.
+# tokens through autograd 286 -> 173 us.  Each function returns None for
+# arguments it does not take; the checks here then follow.  None until the
+# library is loaded, or when the module was not built.
 _native = None
 
 _P = ctypes.c_void_p

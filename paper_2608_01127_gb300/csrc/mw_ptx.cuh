@@ -66,26 +66,45 @@ struct WaitCtl {
 
 // Waits for the phase with the given parity; gives up after the budget (or
 // when another role of the CTA already gave up), records the timeout in the
-// status word and returns false.  Never traps.
+// status word and returns false.  Never traps.  The abort flag and the clock
+// are looked at only every 32nd poll (try_wait itself suspends the thread for
+// a while): a read of the clock before the first one delayed every wait.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtl& ctl) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
-  uint32_t spins = 0;
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
+  uint64_t t0 = 0;
+  for (uint32_t spins = 1; !mbar_try_wait(bar, parity); ++spins) {
+    if ((spins & 31u) != 0u) continue;
     if (*ctl.abort) return false;
-    if (((++spins) & 63u) == 0u && global_timer_ns() - t0 > ctl.budget_ns) {
+    const uint64_t t = global_timer_ns();
+    if (t0 == 0) t0 = t;
+    if (t - t0 > ctl.budget_ns) {
       *ctl.abort = 1;
       atomicOr(ctl.status, kDevTimeout);
       return false;
     }
   }
+  return true;
 }
 
-// Warp-uniform variant: every lane of the warp gets the same answer, so
-// that .sync.aligned tcgen05 instructions after it are never divergent.
+// The same for a whole converged warp: every lane gets the same answer, so
+// that .sync.aligned tcgen05 instructions after it are never divergent.  The
+// loop itself is uniform (a vote a poll): a vote over mbar_wait's answers
+// took 104 cycles for a phase that was complete already, this form 59.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const WaitCtl& ctl) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, ctl));
+  uint64_t t0 = 0;
+  for (uint32_t spins = 1; !__all_sync(0xffffffffu, mbar_try_wait(bar, parity)); ++spins) {
+    if ((spins & 31u) != 0u) continue;
+    const uint64_t t = global_timer_ns();
+    if (t0 == 0) t0 = t;
+    const bool late = t - t0 > ctl.budget_ns;
+    if (__any_sync(0xffffffffu, late || *ctl.abort)) {
+      if (late) {
+        *ctl.abort = 1;
+        atomicOr(ctl.status, kDevTimeout);
+      }
+      return false;
+    }
+  }
+  return true;
 }
 
 // Bounded wait used only on the abort path (lets in-flight copies land
