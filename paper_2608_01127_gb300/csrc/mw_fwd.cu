@@ -712,10 +712,21 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
 }
 
 // Merge of split-KV partials (per row): LSE = ln sum_s exp(LSE_s),
-// O = sum_s exp(LSE_s - LSE) O_s.  One warp per row, 8 rows per block; the
-// blocks after those carry the ring commit cj (one thread per 16-byte piece
-// of a committed row of one head), when there is one.
+// O = sum_s exp(LSE_s - LSE) O_s.  D / 8 lanes per row, 8 columns each, and
+// kCombineRows rows a lane, all of whose loads are issued before the first is
+// used (S splits, 2 to 4; S = 0: any number, one after another): the partials
+// come from L2, so bytes in flight bound it (a warp a row with one 16-byte load
+// a split: streaming step of 12 heads of 64, three splits, 15.9 us a step, this
+// form 14.3; 16 heads of 128, 4 x 880 rows, two splits, combine alone 17.4 ->
+// 15.6 us).  The blocks after those carry the
+// ring commit cj (one thread per 16-byte piece of a committed row of one
+// head), when there is one.
+constexpr int kCombineRows = 2;
 template <int D>
+constexpr int combine_block_rows() {
+  return kCombineRows * 256 / (D / 8);
+}
+template <int D, int S>
 __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ o_part,
                                                       const float* __restrict__ lse_part,
                                                       __nv_bfloat16* __restrict__ o,
@@ -724,7 +735,9 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
                                                       const CommitJob cj) {
   pdl_wait();     // the forward's partials (and its reads of the ring) are complete
   pdl_trigger();  // the next step's forward may start its setup meanwhile
-  const int combine_blocks = (n_rows + 7) / 8;
+  constexpr int G = D / 8;  // lanes per row
+  constexpr int kBlockRows = combine_block_rows<D>();
+  const int combine_blocks = (n_rows + kBlockRows - 1) / kBlockRows;
   if (static_cast<int>(blockIdx.x) >= combine_blocks) {
     const long long idx =
         static_cast<long long>(blockIdx.x - combine_blocks) * blockDim.x + threadIdx.x;
@@ -734,54 +747,73 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
     return;
   }
   const int d_io = (D == 64) ? D : d_io_arg;  // padded head dims use the 128-wide kernels
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n_rows) return;
-  constexpr int PER = D / 32;
-  float acc[PER];
+  const int sub = threadIdx.x % G;
+  // (the multiples of 8 columns past the caller's hold nothing)
+  if (8 * sub >= d_io) return;
+  const int row0 = blockIdx.x * kBlockRows + threadIdx.x / G;
+  constexpr int kStep = 256 / G;  // rows between a lane's rows
+  constexpr int NS = S > 0 ? S : 1;
+  const size_t split_stride = static_cast<size_t>(n_rows) * D;
+  float ls[kCombineRows][NS];
+  float4 x[kCombineRows][NS][2];
+  auto load = [&](int r, int k, int s) {
+    const int row = row0 + r * kStep;
+    const float4* src =
+        reinterpret_cast<const float4*>(o_part + s * split_stride + static_cast<size_t>(row) * D) + 2 * sub;
+    x[r][k][0] = src[0];
+    x[r][k][1] = src[1];
+  };
+  if constexpr (S > 0) {
 #pragma unroll
-  for (int k = 0; k < PER; ++k) acc[k] = 0.f;
-  float wsum = 0.f, m = -INFINITY;
-  using Vec = typename std::conditional<PER == 4, float4, float2>::type;  // a lane's columns
-  // a split whose LSE is -inf saw no key of the row: its O part is skipped
-  // (never multiplied: it may hold anything)
-  auto add = [&](float ls, const Vec& x) {
-    const float w = ls == -INFINITY ? 0.f : __expf(ls - m);
-    wsum += w;
-    if (w > 0.f) {
-      acc[0] += w * x.x;
-      acc[1] += w * x.y;
-      if constexpr (PER == 4) {
-        acc[2] += w * x.z;
-        acc[3] += w * x.w;
+    for (int r = 0; r < kCombineRows; ++r)
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if (row0 + r * kStep < n_rows) {
+          ls[r][s] = lse_part[static_cast<size_t>(s) * n_rows + row0 + r * kStep];
+          load(r, s, s);
+        }
+  }
+#pragma unroll
+  for (int r = 0; r < kCombineRows; ++r) {
+    const int row = row0 + r * kStep;
+    if (row >= n_rows) return;
+    float acc[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+    float wsum = 0.f, m = -INFINITY;
+    // a split whose LSE is -inf saw no key of the row: its O part is skipped
+    // (never multiplied: it may hold anything)
+    auto add = [&](float l, const float4 (&v)[2]) {
+      const float w = l == -INFINITY ? 0.f : __expf(l - m);
+      wsum += w;
+      if (w > 0.f) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          acc[4 * h] += w * v[h].x;
+          acc[4 * h + 1] += w * v[h].y;
+          acc[4 * h + 2] += w * v[h].z;
+          acc[4 * h + 3] += w * v[h].w;
+        }
+      }
+    };
+    if constexpr (S > 0) {
+#pragma unroll
+      for (int s = 0; s < S; ++s) m = fmaxf(m, ls[r][s]);
+#pragma unroll
+      for (int s = 0; s < S; ++s) add(ls[r][s], x[r][s]);
+    } else {
+      for (int s = 0; s < splits; ++s) m = fmaxf(m, lse_part[static_cast<size_t>(s) * n_rows + row]);
+      for (int s = 0; s < splits; ++s) {
+        load(r, 0, s);
+        add(lse_part[static_cast<size_t>(s) * n_rows + row], x[r][0]);
       }
     }
-  };
-  const Vec* src0 = reinterpret_cast<const Vec*>(o_part + static_cast<size_t>(row) * D) + lane;
-  const size_t split_stride = static_cast<size_t>(n_rows) * D / PER;  // in Vec
-  if (splits == 2) {
-    // the usual case: both LSEs and both O parts requested at once (one
-    // memory round trip instead of four)
-    const float l0 = lse_part[row], l1 = lse_part[static_cast<size_t>(n_rows) + row];
-    const Vec x0 = src0[0], x1 = src0[split_stride];
-    m = fmaxf(l0, l1);
-    add(l0, x0);
-    add(l1, x1);
-  } else {
-    for (int s = 0; s < splits; ++s) m = fmaxf(m, lse_part[static_cast<size_t>(s) * n_rows + row]);
-    for (int s = 0; s < splits; ++s)
-      add(lse_part[static_cast<size_t>(s) * n_rows + row], src0[s * split_stride]);
+    const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
+    *reinterpret_cast<uint4*>(o + static_cast<size_t>(row) * d_io + 8 * sub) =
+        make_uint4(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv),
+                   pack_bf16x2(acc[4] * inv, acc[5] * inv), pack_bf16x2(acc[6] * inv, acc[7] * inv));
+    if (lse && sub == 0) lse[row] = wsum > 0.f ? m + __logf(wsum) : -INFINITY;
   }
-  const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-  __nv_bfloat16* dst = o + static_cast<size_t>(row) * d_io + lane * PER;
-  if (lane * PER < d_io) {  // d_io is a multiple of 8, so a lane's PER columns are all in range
-    if constexpr (PER == 4)
-      *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(acc[0] * inv, acc[1] * inv),
-                                                  pack_bf16x2(acc[2] * inv, acc[3] * inv));
-    else
-      *reinterpret_cast<uint32_t*>(dst) = pack_bf16x2(acc[0] * inv, acc[1] * inv);
-  }
-  if (lse && lane == 0) lse[row] = wsum > 0.f ? m + __logf(wsum) : -INFINITY;
 }
 
 template <int D, int DM, bool ROPE, bool SPLIT>
@@ -841,15 +873,23 @@ cudaError_t launch_combine(int d, int d_io, const float* o_part, const float* ls
                            const CommitJob& cj, cudaStream_t s) {
   const int n_rows = BH * rows;
   const long long commit_pieces = static_cast<long long>(cj.rows) * (cj.d / 8) * cj.BH;
-  const long long blocks = (n_rows + 7) / 8 + (commit_pieces + 255) / 256;
+  const int block_rows = d == 64 ? combine_block_rows<64>() : combine_block_rows<128>();
+  const long long blocks = (n_rows + block_rows - 1) / block_rows + (commit_pieces + 255) / 256;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;
   pdl_config(cfg, attr, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s);
+  auto launch = [&](auto kernel) {
+    return cudaLaunchKernelEx(&cfg, kernel, o_part, lse_part, o, lse, splits, n_rows, d_io, cj);
+  };
   if (d == 64)
-    return cudaLaunchKernelEx(&cfg, combine_kernel<64>, o_part, lse_part, o, lse, splits, n_rows,
-                              d_io, cj);
-  return cudaLaunchKernelEx(&cfg, combine_kernel<128>, o_part, lse_part, o, lse, splits, n_rows,
-                            d_io, cj);
+    return launch(splits == 2   ? combine_kernel<64, 2>
+                  : splits == 3 ? combine_kernel<64, 3>
+                  : splits == 4 ? combine_kernel<64, 4>
+                                : combine_kernel<64, 0>);
+  return launch(splits == 2   ? combine_kernel<128, 2>
+                : splits == 3 ? combine_kernel<128, 3>
+                : splits == 4 ? combine_kernel<128, 4>
+                              : combine_kernel<128, 0>);
 }
 
 }  // namespace mw
