@@ -12,27 +12,29 @@
 namespace mw {
 namespace {
 
-constexpr int kQkvTokens = 32;  // tokens per CTA
+constexpr int kQkvTokens = 32;  // at most, per CTA
 constexpr int kMaxPairs = kMaxRopePairs;
-constexpr int kUnroll = 4;      // heads whose 16-byte pieces are in flight at once
+constexpr int kMaxUnroll = 6;
 
-// grid.x: (b, block of kQkvTokens tokens); grid.y: groups of heads_per_block
+// grid.x: (b, block of `tokens` tokens); grid.y: groups of heads_per_block
 // heads.  A thread owns one (token, 16-byte piece) of the block, fixed for
 // the whole kernel, and walks Q, K, V and the group's heads with plain
-// strides; each warp reads whole 128-byte row segments and writes 512
-// contiguous bytes.
+// strides, UNROLL heads' pieces in flight at once; each warp reads whole row
+// segments and writes contiguous bytes.
+template <int UNROLL>
 __global__ void __launch_bounds__(256) qkv_rope_kernel(const __nv_bfloat16* __restrict__ qkv,
                                                        __nv_bfloat16* __restrict__ q,
                                                        __nv_bfloat16* __restrict__ k,
                                                        __nv_bfloat16* __restrict__ v, int N, int H,
-                                                       int d, int rope_dims, int heads_per_block,
+                                                       int d, int tokens, int rope_dims,
+                                                       int heads_per_block,
                                                        const RopeFreq omega, int per_frame,
                                                        int first_frame) {
   __shared__ float2 table[kQkvTokens * kMaxPairs];  // (cos, sin) per (frame, pair)
-  const int n_tb = (N + kQkvTokens - 1) / kQkvTokens;
+  const int n_tb = (N + tokens - 1) / tokens;
   const int b = blockIdx.x / n_tb;
-  const int t0 = (blockIdx.x % n_tb) * kQkvTokens;
-  const int nt = min(kQkvTokens, N - t0);
+  const int t0 = (blockIdx.x % n_tb) * tokens;
+  const int nt = min(tokens, N - t0);
   const int h0 = blockIdx.y * heads_per_block;
   const int h1 = min(H, h0 + heads_per_block);
   const int pairs = rope_dims / 2;
@@ -63,14 +65,14 @@ __global__ void __launch_bounds__(256) qkv_rope_kernel(const __nv_bfloat16* __re
     for (int which = 0; which < 3; ++which) {
       __nv_bfloat16* out = which == 0 ? q : which == 1 ? k : v;
       const bool turn = which < 2 && np > 0;
-      for (int h = h0; h < h1; h += kUnroll) {
-        uint4 x[kUnroll];
+      for (int h = h0; h < h1; h += UNROLL) {
+        uint4 x[UNROLL];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u)
+        for (int u = 0; u < UNROLL; ++u)
           if (h + u < h1)
             x[u] = *reinterpret_cast<const uint4*>(src + static_cast<size_t>(which * H + h + u) * d);
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < UNROLL; ++u) {
           if (h + u >= h1) continue;
           if (turn) {
             x[u].x = rope_turn(x[u].x, cs[0]);
@@ -92,15 +94,36 @@ cudaError_t launch_qkv_rope(const __nv_bfloat16* qkv, __nv_bfloat16* q, __nv_bfl
                             const RopeFreq& omega, int per_frame, int first_frame,
                             cudaStream_t s) {
   if (B == 0 || N == 0 || H == 0) return cudaSuccess;
-  const long long tb = static_cast<long long>(B) * ((N + kQkvTokens - 1) / kQkvTokens);
+  // as many tokens as fill the 256 threads (d = 128: twice), so that no pass
+  // over the block is mostly idle: 32 tokens of 72 channels are 288 pieces
+  const int pieces = d / 8;
+  const int tokens = pieces == 16 ? kQkvTokens : 256 / pieces;
+  const long long tb = static_cast<long long>(B) * ((N + tokens - 1) / tokens);
   // halve the heads per CTA until the grid holds enough CTAs to fill every SM
   // a few times over (the per-CTA (cos, sin) table is then amortised over as
   // many heads as the size allows)
   int hb = H;
   while (hb > 1 && tb * ((H + hb - 1) / hb) < 1216) hb = (hb + 1) / 2;
+  // heads in flight: the fewest equal batches of up to six (12 heads of 64,
+  // 2 x 14080 tokens, six heads a CTA: one batch of six 41.7 us, four and two
+  // 42.8; 16 heads of 128, eight a CTA: four and four 73 us, six and two 79).
+  // With both rules, a call of 16 heads of 72: 41.8 -> 35.9 us, 7 heads of 80:
+  // 23.1 -> 16.8 us, 24 heads of 64: 66.3 -> 61.4 us
+  const int batches = (hb + kMaxUnroll - 1) / kMaxUnroll;
+  const int unroll = (hb + batches - 1) / batches;
   const dim3 grid(static_cast<unsigned>(tb), static_cast<unsigned>((H + hb - 1) / hb));
-  qkv_rope_kernel<<<grid, 256, 0, s>>>(qkv, q, k, v, N, H, d, rope_dims, hb, omega, per_frame,
-                                       first_frame);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, 256, 0, s>>>(qkv, q, k, v, N, H, d, tokens, rope_dims, hb, omega, per_frame,
+                                first_frame);
+  };
+  switch (unroll) {
+    case 1: launch(qkv_rope_kernel<1>); break;
+    case 2: launch(qkv_rope_kernel<2>); break;
+    case 3: launch(qkv_rope_kernel<3>); break;
+    case 4: launch(qkv_rope_kernel<4>); break;
+    case 5: launch(qkv_rope_kernel<5>); break;
+    default: launch(qkv_rope_kernel<6>); break;
+  }
   return cudaGetLastError();
 }
 

@@ -1,0 +1,36 @@
+"""Kernel variants and launch shapes that are chosen by size: each at the edges
+of the sizes that choose it, against the oracle or a plain copy."""
+import importlib
+
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mw():
+    return importlib.import_module("paper_2608_01127_gb300")
+
+
+@pytest.mark.parametrize("H", [1, 2, 3, 4, 5, 6, 7, 11, 13])  # heads in flight: 1 to 6
+@pytest.mark.parametrize("d,N", [(64, 33), (72, 28), (72, 29), (80, 26), (88, 22), (96, 43),
+                                 (104, 20), (112, 17), (120, 35), (128, 31)])
+def test_qkv_split_token_blocks(mw, H, d, N):
+    """A block of tokens fills the threads once (twice at d = 128): at, below
+    and above a block's size; V and unrotated channels bit for bit, rotated
+    ones as the oracle rounds them (one bf16 ulp, plus what the 1e-6 rad of the
+    angle leaves where the two products cancel)."""
+    g = torch.Generator().manual_seed(d * 100 + N + H)
+    qkv = torch.randn(2, N, 3, H, d, generator=g).to(torch.bfloat16)
+    rope = d // 2 // 2 * 2 - 2  # ends inside a 16-byte piece for most d
+    q, k, v = mw.mw_qkv_rope_split(qkv.cuda(), rope, 1e4, 9, 5)
+    ref = oracle.qkv_split_rope(qkv, rope, 1e4, 9, 5)
+    assert torch.equal(v.cpu(), qkv[:, :, 2].permute(0, 2, 1, 3))
+    for got, want in ((q, ref[0]), (k, ref[1])):
+        got = got.cpu().double()
+        assert torch.equal(got[..., rope:], want[..., rope:].double())
+        err = (got - want).abs()
+        assert bool((err <= want.abs() * 2.0 ** -7 + 2.0 ** -16).all())
