@@ -245,6 +245,19 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
     *abort_flag = 0;
     fence_mbar_init();
   }
+  // descriptors (kernel parameters, so they may be read before the previous
+  // kernel ends): in the setup where a launch has few key tiles a CTA (rolling
+  // step 58.9 -> 57.8 us); the unsplit forward measured 0.2% slower that way
+  auto prefetch_maps = [&]() {
+    prefetch_tmap(&tm_q);
+    prefetch_tmap(&tm_k);
+    prefetch_tmap(&tm_v);
+    if constexpr (SPLIT) {
+      prefetch_tmap(&tm_kr);
+      prefetch_tmap(&tm_vr);
+    }
+  };
+  if (SPLIT && warp == 8 && lane == 0) prefetch_maps();
   if (warp == 9) {
     tmem_alloc(tmem_slot, 512);
     tmem_relinquish();
@@ -277,9 +290,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
   if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0 && n_local > 0) {
-      prefetch_tmap(&tm_q);
-      prefetch_tmap(&tm_k);
-      prefetch_tmap(&tm_v);
+      if (!SPLIT) prefetch_maps();
       bool q_issued = false;
       if (!p.debug_skip_q) {
         mbar_arrive_expect_tx(q_full, QT * L::TILE_BYTES);
