@@ -57,6 +57,11 @@ mw_status ok() {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Rows of d bf16 from p all start at multiples of 32 bytes.
+bool wide_rows(const void* p, int d) {
+  return (reinterpret_cast<uintptr_t>(p) & 31u) == 0 && d % 16 == 0;
+}
+
 mw_status check_ptr(const void* p, const char* name) {
   if (p == nullptr) return fail(MW_ERR_INVALID_ARG, "%s is NULL", name);
   if (!aligned16(p)) return fail(MW_ERR_INVALID_ARG, "%s is not 16-byte aligned", name);
@@ -463,6 +468,7 @@ mw_status fwd_common(const void* q, const void* k, const void* v, const void* kr
   p.num_splits = splits;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.o = static_cast<__nv_bfloat16*>(o);
+  p.wide_out = wide_rows(o, d);
   p.lse = lse;
   p.status = status;
   p.budget_ns = budget_ns();
@@ -649,6 +655,7 @@ mw_status mw_bca_bwd_stage(int stage, const void* q, const void* k, const void* 
     p.dq_acc = dq_acc;
     p.dk = static_cast<__nv_bfloat16*>(dk);
     p.dv = static_cast<__nv_bfloat16*>(dv);
+    p.wide_out = wide_rows(dk, d) && wide_rows(dv, d);
     p.status = status;
     p.budget_ns = budget_ns();
     p.debug_skip_q = static_cast<int>(g_opt_skip_q);

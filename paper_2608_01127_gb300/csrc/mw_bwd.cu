@@ -681,14 +681,10 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
           for (int k = 0; k < 32; ++k) r[k] = 0u;
         }
         if (k_valid && 32 * c < d_io) {
-          const int n16 = min(4, (d_io - 32 * c) / 8);
-          uint4* dst = reinterpret_cast<uint4*>(out + row_off + 32 * c);
+          float v[32];
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (k < n16) dst[k] = make_uint4(pack_bf16x2(__uint_as_float(r[8 * k]) * mul, __uint_as_float(r[8 * k + 1]) * mul),
-                                pack_bf16x2(__uint_as_float(r[8 * k + 2]) * mul, __uint_as_float(r[8 * k + 3]) * mul),
-                                pack_bf16x2(__uint_as_float(r[8 * k + 4]) * mul, __uint_as_float(r[8 * k + 5]) * mul),
-                                pack_bf16x2(__uint_as_float(r[8 * k + 6]) * mul, __uint_as_float(r[8 * k + 7]) * mul));
+          for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]) * mul;
+          store_row32(out + row_off + 32 * c, v, min(4, (d_io - 32 * c) / 8), p.wide_out);
         }
       }
     }

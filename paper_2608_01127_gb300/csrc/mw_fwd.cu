@@ -263,8 +263,10 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
     tmem_relinquish();
   }
   if constexpr (L::ONES_BYTES > 0) {
-    uint32_t* ones = reinterpret_cast<uint32_t*>(smem + L::OFF_ONES);
-    for (int k = threadIdx.x; k < L::ONES_BYTES / 4; k += L::THREADS) ones[k] = 0x3F803F80u;  // bf16 1.0
+    uint4* ones = reinterpret_cast<uint4*>(smem + L::OFF_ONES);
+    const uint32_t one2 = 0x3F803F80u;  // bf16 1.0 twice
+    for (int k = threadIdx.x; k < L::ONES_BYTES / 16; k += L::THREADS)
+      ones[k] = make_uint4(one2, one2, one2, one2);
     fence_proxy_async_smem();  // read by the tensor core (async proxy)
   }
   tc_fence_before();
@@ -661,13 +663,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
           // the 128-wide kernel serves padded head dims
           const int d_io = (D == 64) ? D : p.d_io;
           if (32 * c >= d_io) continue;
-          const int n16 = min(4, (d_io - 32 * c) / 8);
-          uint4* dst = reinterpret_cast<uint4*>(p.o + row_off * d_io + 32 * c);
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (k < n16) dst[k] = make_uint4(pack_bf16x2(v[8 * k], v[8 * k + 1]), pack_bf16x2(v[8 * k + 2], v[8 * k + 3]),
-                                pack_bf16x2(v[8 * k + 4], v[8 * k + 5]),
-                                pack_bf16x2(v[8 * k + 6], v[8 * k + 7]));
+          store_row32(p.o + row_off * d_io + 32 * c, v, min(4, (d_io - 32 * c) / 8), p.wide_out);
         } else {
           // never taken (the launcher picks SPLIT for several splits), but
           // with this row-per-thread form of the partials here the compiler

@@ -52,6 +52,7 @@ struct FwdParams {
   int num_splits;   // 1: write bf16 O + LSE; >1: fp32 partials for the combine
   float scale_log2; // softmax scale * log2(e)
   __nv_bfloat16* o;
+  bool wide_out;    // every row of o starts at a multiple of 32 bytes
   float* lse;       // nullable
   float* o_part;    // [splits, BH, rows_q, d]
   float* lse_part;  // [splits, BH, rows_q]
@@ -74,6 +75,7 @@ struct BwdParams {
   float* dq_acc;       // [BH, N_pad, d] fp32
   __nv_bfloat16* dk;
   __nv_bfloat16* dv;
+  bool wide_out;       // every row of both starts at a multiple of 32 bytes
   unsigned* status;
   unsigned long long budget_ns;
   int debug_skip_q;  // test hook: never load Q, so the first S^T wait expires

@@ -34,3 +34,28 @@ def test_qkv_split_token_blocks(mw, H, d, N):
         assert torch.equal(got[..., rope:], want[..., rope:].double())
         err = (got - want).abs()
         assert bool((err <= want.abs() * 2.0 ** -7 + 2.0 ** -16).all())
+
+
+@pytest.mark.parametrize("d", [64, 72, 80, 96, 120, 128])
+def test_output_rows_at_16_and_32_bytes(mw, d):
+    """O, dK and dV rows go out as 32-byte stores where every row starts at a
+    multiple of 32 bytes, else as 16-byte ones: the same bits either way, and
+    nothing written beyond the outputs."""
+    B, H, N, T = 1, 2, 150, 50
+    g = torch.Generator("cuda").manual_seed(d)
+    q, k, v, do = (torch.randn(B, H, N, d, generator=g, device="cuda").to(torch.bfloat16)
+                   for _ in range(4))
+    n = B * H * N * d
+    results = []
+    for shift in (16, 8):  # in elements: 32 and 16 bytes
+        bufs = [torch.full((n + 64,), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(4)]
+        o, dq, dk, dv = (b[shift:shift + n].view(B, H, N, d) for b in bufs)
+        _, lse = mw.mw_bca_fwd(q, k, v, T, out=(o, torch.empty(B, H, N, device="cuda")))
+        mw.mw_bca_bwd(q, k, v, o, lse, do, T, out=(dq, dk, dv))
+        for b in bufs:
+            assert bool((b[:shift] == 7).all()) and bool((b[shift + n:] == 7).all())
+        results.append((o, dk, dv, lse))
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
+    o_ref, _ = oracle.fwd(q.cpu(), k.cpu(), v.cpu(), T, d ** -0.5)
+    assert float((results[0][0].double().cpu() - o_ref).norm() / o_ref.norm()) <= 5e-3
