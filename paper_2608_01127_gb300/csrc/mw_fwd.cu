@@ -10,15 +10,17 @@
 // Roles (384 threads):
 //   warps 0-3 / 4-7  softmax of query tile 0 / 1 (one thread per row = TMEM lane)
 //   warp 8           TMA producer (Q once, then K/V tiles through a ring of stages)
-//   warp 9           tcgen05 issuer (S = Q K^T into TMEM, O += P V with P in TMEM)
-//   warps 10-11      RoPE re-shift of the sink anchor's key tiles in shared
+//   warp 9           tcgen05 issuer (S = Q K^T into TMEM, O += P V with P in TMEM);
+//                    d = 64: of query tile 0, and warp 10 of query tile 1
+//   the rest of 10-11 RoPE re-shift of the sink anchor's key tiles in shared
 //                    memory when it is enabled; with 80-wide MMAs on the
 //                    128-wide tiles (and no re-shift) the ones columns of V;
 //                    otherwise idle (they complete warpgroup 2 for the
 //                    register re-split)
-// TMEM (512 columns): S_t at column 128 t (P_t, bf16, overwrites its first 64
-// columns), O_t at 256 + OW t (OW = the MMA width, plus 16 columns where the
-// PV MMA also sums P through ones in V).
+// TMEM (512 columns): S_t at column 128 t, O_t at 256 + OW t (OW = the MMA
+// width, plus 16 columns where the PV MMA also sums P through ones in V).
+// P_t, bf16, overwrites the first 64 columns of S_t; where there is room, only
+// its first half does, and the second lies after the O columns.
 // CTA order: groups of heads of about three waves of CTAs, one group after
 // another; in a group the longest query blocks first.
 #include <type_traits>
@@ -33,7 +35,7 @@ namespace {
 // columns past the caller's zero-filled by TMA); DM <= D: the columns the
 // MMAs cover (QK^T reduces over DM, O has DM columns), 80 for head dims up
 // to 80 on the 128-wide tiles
-template <int D, int DM = D, bool ROPE = false>
+template <int D, int DM = D, bool ROPE = false, bool SPLIT = false>
 struct FwdLayout {
   static_assert(DM % 16 == 0 && DM <= D, "MMA width");
   static constexpr int QT = kFwdQTiles;
@@ -49,7 +51,7 @@ struct FwdLayout {
   // d = 64: the ones are a region of their own, reached through each stage
   // descriptor's leading-byte offset.  80-wide MMAs on the 128-wide tiles:
   // the ones go into columns 80..95 of each V tile (which TMA fills with
-  // zeros), written by warps 10-11 after every load; with the RoPE re-shift
+  // zeros), written by the helper warps after every load; with the RoPE re-shift
   // those warps are busy and the softmax sums P itself.
   static constexpr bool ONES_IN_V = (D == 128 && DM == 80 && !ROPE);
   static constexpr bool SUM_MMA = (D == 64) || ONES_IN_V;
@@ -63,11 +65,34 @@ struct FwdLayout {
   static constexpr int ROPE_WARP_BYTES = (D / 2) * 8;
   static constexpr int ROPE_BYTES = 2 * ROPE_WARP_BYTES;
   static constexpr int OFF_BAR = OFF_ROPE + ROPE_BYTES;
-  static constexpr int NBAR = 1 + 6 * STAGES + 3 * QT + 1;
+  // P of a key tile's last 64 keys in columns of its own, where TMEM has room
+  // (d = 64, and 80-wide MMAs): S is then free once the PV of the first 64
+  // keys is issued, and the next tile's QK^T runs before the second half of P
+  // is there, so that both tiles' softmax warps work all the time instead of
+  // in turn (P over S as a whole leaves each tile's softmax waiting for its own
+  // PV and QK^T).  d = 64, 24 heads x 16 x 880: 613 us before, 594 with the
+  // early exponentials below alone, 568 with both and an issuer per tile; 16
+  // heads of 72: 445, 438 and 436 us (with one issuer).  A split key range is
+  // a handful of tiles a CTA, which the chain through the first and the last
+  // of them dominates: it gains nothing (one step against 8 chunks of 880, 12
+  // heads of 64: 30.3 us against 30.6 with it; 16 of 72: 46.0 against 47.6).
+  static constexpr bool SPLIT_P = !SPLIT && 256 + OW * QT + 32 * QT <= 512;
+  // MMA-issuing warps: at d = 64 one per query tile (warps 9 and 10), since a
+  // step's waits and commits take an issuer about as long as its MMAs take the
+  // tensor core, whose queue is only two instructions deep (601 us with one).
+  // The 80-wide kernels need two warps for the ones columns of V (495 us with
+  // two issuers and one helper).
+  static constexpr int ISSUERS = D == 64 && SPLIT_P ? QT : 1;
+  static constexpr int HELPERS = 3 - ISSUERS;  // the warps after the issuers
+  static constexpr int NBAR = 1 + 6 * STAGES + (SPLIT_P ? 4 : 3) * QT + 1;
   static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
   static constexpr int BYTES = OFF_MISC + 16;
   static constexpr uint32_t S_COL(int t) { return 128u * t; }
   static constexpr uint32_t O_COL(int t) { return 256u + OW * t; }
+  // P of the first and of the last 64 keys of a tile
+  static constexpr uint32_t P_COL(int t, int half) {
+    return half == 0 ? S_COL(t) : SPLIT_P ? 256u + OW * QT + 32u * t : S_COL(t) + 32u;
+  }
   static constexpr int THREADS = 384;
   // registers per thread after the re-split: softmax warpgroups 0-1 get
   // more, warpgroup 2 (TMA, MMA, RoPE or idle warps) less; 2*128*S + 128*C
@@ -126,7 +151,7 @@ __device__ __forceinline__ TileSrc tile_src(const Segs& g, int j) {
   return s;
 }
 
-// ROPE: the cache form with the RoPE re-shift of the sink anchor (warps 10-11
+// ROPE: the cache form with the RoPE re-shift of the sink anchor (the helper warps
 // turn its key tiles before the MMAs read them); the training and plain
 // cache forms are compiled without it.  SPLIT: the key range is one of
 // several (p.num_splits > 1), O goes out as fp32 partials through TMA
@@ -139,7 +164,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
                    const __grid_constant__ CUtensorMap tm_vr, const __grid_constant__ CUtensorMap tm_ks,
                    const __grid_constant__ CUtensorMap tm_vs, const __grid_constant__ CUtensorMap tm_op,
                    const __grid_constant__ FwdParams p, const __grid_constant__ RopeFreq rope_om) {
-  using L = FwdLayout<D, DM, ROPE>;
+  using L = FwdLayout<D, DM, ROPE, SPLIT>;
   constexpr int QT = L::QT;
   constexpr int NS = L::STAGES;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -196,7 +221,8 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
   uint64_t* s_full = v_rdy + NS;
   uint64_t* p_full = s_full + QT;
   uint64_t* p_half = p_full + QT;  // first 64 keys of P in TMEM
-  uint64_t* o_full = p_half + QT;
+  uint64_t* pv_done = p_half + QT;  // SPLIT_P: the PV of a key tile is done
+  uint64_t* o_full = pv_done + (L::SPLIT_P ? QT : 0);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 4);
 
@@ -226,22 +252,24 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
   const int j1 = (int)((long long)(split + 1) * n_all / p.num_splits);
   const int n_local = j1 - j0;
 
+  const int n_issuers = L::ISSUERS == 1 ? 1 : min(L::ISSUERS, qt_n);  // that have a query tile
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     for (int s = 0; s < NS; ++s) {
       mbar_init(&k_full[s], 1);
-      mbar_init(&k_empty[s], 1);
+      mbar_init(&k_empty[s], n_issuers);
       mbar_init(&v_full[s], 1);
-      mbar_init(&v_empty[s], 1);
-      mbar_init(&k_rdy[s], 2);
-      mbar_init(&v_rdy[s], 2);
+      mbar_init(&v_empty[s], n_issuers);
+      mbar_init(&k_rdy[s], L::HELPERS);
+      mbar_init(&v_rdy[s], L::HELPERS);
     }
     for (int t = 0; t < QT; ++t) {
       mbar_init(&s_full[t], 1);
       mbar_init(&p_full[t], 4);
       mbar_init(&p_half[t], 4);
+      if constexpr (L::SPLIT_P) mbar_init(&pv_done[t], 1);
     }
-    mbar_init(o_full, 1);
+    mbar_init(o_full, n_issuers);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -331,8 +359,8 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
           drain_wait(&v_full[i % NS], (i / NS) & 1, p.budget_ns);
       }
     }
-  } else if (warp == 9) {
-    // ------------------------------------------------------------ MMA issuer (whole warp)
+  } else if (warp == 9 || (L::ISSUERS > 1 && warp == 10)) {
+    // ------------------------------------------------------------ MMA issuers (whole warps)
     if (n_local > 0) {
       constexpr uint32_t idesc_qk = idesc_bf16_f32(128, 128, false, false);
       constexpr uint32_t idesc_pv = idesc_bf16_f32(128, L::OW, false, true);
@@ -360,67 +388,126 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
 #pragma unroll
         for (int k4 = 0; k4 < 4; ++k4) {
           const int kk = 4 * half + k4;
-          umma_ts(tmem + L::O_COL(t), tmem + L::S_COL(t) + kk * 8, sdesc_add(vb, kk * 2048),
+          umma_ts(tmem + L::O_COL(t), tmem + L::P_COL(t, half) + k4 * 8, sdesc_add(vb, kk * 2048),
                   idesc_pv, (acc || kk > 0) ? 1u : 0u);
         }
       };
 
       bool ok = warp_wait(q_full, 0, ctl);
       tc_fence_after();
-      for (int i = 0; ok && i < n_local; ++i) {
-        const int st = i % NS;
-        const uint32_t ph = (i / NS) & 1;
-        const int stp = (i + NS - 1) % NS;
-        const uint32_t php = ((i - 1) / NS) & 1;
-        // with the re-shift, a sink tile is read once warps 10-11 have turned it
-        const bool turned = ROPE && j0 + i < g.nS;
-        if (!(ok = warp_wait(turned ? &k_rdy[st] : &k_full[st], ph, ctl))) break;
-        tc_fence_after();
-        // unrolled over the compile-time tile count, so every descriptor
-        // offset stays a constant (a runtime trip count here slows the whole
-        // forward by ~8%: the issuing code must never pause)
+      if constexpr (L::SPLIT_P) {
+        // K tile i in shared memory (with the re-shift, a sink tile is read
+        // once the helper warps have turned it)
+        auto wait_k = [&](int i) {
+          const int st = i % NS;
+          return warp_wait(ROPE && j0 + i < g.nS ? &k_rdy[st] : &k_full[st], (i / NS) & 1, ctl);
+        };
+        // query tiles [first, last): one issuer's, or all of them
+        auto issue = [&](auto first, auto last) {
+          constexpr int T0 = decltype(first)::value, T1 = decltype(last)::value;
+          if (T0 >= qt_n) return;
+          if (ok && (ok = wait_k(0))) {
+            tc_fence_after();
 #pragma unroll
-        for (int t = 0; t < QT; ++t) {
-          if (t >= qt_n) break;
-          if (i > 0) {
-            // PV of the first 64 keys while the softmax warps store the rest of P
-            if (!(ok = warp_wait(&p_half[t], (i - 1) & 1, ctl))) break;
-            if (t == 0 && !(ok = warp_wait(L::ONES_IN_V ? &v_rdy[stp] : &v_full[stp], php, ctl))) break;
-            tc_fence_after();
-            issue_pv(t, stp, i - 1 > 0, 0);
-            if (!(ok = warp_wait(&p_full[t], (i - 1) & 1, ctl))) break;
-            tc_fence_after();
-            issue_pv(t, stp, true, 1);
+            for (int t = T0; t < T1; ++t) {
+              if (t >= qt_n) break;
+              issue_qk(t, 0);
+              umma_commit(&s_full[t]);
+            }
+            umma_commit(&k_empty[0]);
           }
-          issue_qk(t, st);
-          umma_commit(&s_full[t]);
-        }
-        if (!ok) break;
-        umma_commit(&k_empty[st]);
-        if (i > 0) umma_commit(&v_empty[stp]);
-      }
-      if (ok) {
-        const int il = n_local - 1;
-        const int stl = il % NS;
+          for (int i = 0; ok && i < n_local; ++i) {
+            const int st = i % NS;
+            const int st1 = (i + 1) % NS;
+            const bool more = i + 1 < n_local;
+            if (more && !(ok = wait_k(i + 1))) break;
+            if (!(ok = warp_wait(L::ONES_IN_V ? &v_rdy[st] : &v_full[st], (i / NS) & 1, ctl))) break;
 #pragma unroll
-        for (int t = 0; t < QT; ++t) {
-          if (!ok || t >= qt_n) break;
-          if (!(ok = warp_wait(&p_half[t], il & 1, ctl))) break;
-          if (t == 0 && !(ok = warp_wait(L::ONES_IN_V ? &v_rdy[stl] : &v_full[stl], (il / NS) & 1, ctl)))
-            break;
+            for (int t = T0; t < T1; ++t) {
+              if (t >= qt_n) break;
+              if (!(ok = warp_wait(&p_half[t], i & 1, ctl))) break;
+              tc_fence_after();
+              issue_pv(t, st, i > 0, 0);
+              if (more) {
+                issue_qk(t, st1);
+                umma_commit(&s_full[t]);
+              }
+              if (!(ok = warp_wait(&p_full[t], i & 1, ctl))) break;
+              tc_fence_after();
+              issue_pv(t, st, true, 1);
+              umma_commit(&pv_done[t]);
+            }
+            if (!ok) break;
+            if (more) umma_commit(&k_empty[st1]);
+            umma_commit(&v_empty[st]);
+          }
+          if (ok) umma_commit(o_full);
+        };
+        if constexpr (L::ISSUERS == 1) {
+          issue(std::integral_constant<int, 0>{}, std::integral_constant<int, QT>{});
+        } else {
+          static_assert(QT == 2, "an issuer for each of two query tiles");
+          if (warp == 9)
+            issue(std::integral_constant<int, 0>{}, std::integral_constant<int, 1>{});
+          else
+            issue(std::integral_constant<int, 1>{}, std::integral_constant<int, 2>{});
+        }
+      } else {
+        for (int i = 0; ok && i < n_local; ++i) {
+          const int st = i % NS;
+          const uint32_t ph = (i / NS) & 1;
+          const int stp = (i + NS - 1) % NS;
+          const uint32_t php = ((i - 1) / NS) & 1;
+          // with the re-shift, a sink tile is read once the helper warps have turned it
+          const bool turned = ROPE && j0 + i < g.nS;
+          if (!(ok = warp_wait(turned ? &k_rdy[st] : &k_full[st], ph, ctl))) break;
           tc_fence_after();
-          issue_pv(t, stl, il > 0, 0);
-          if (!(ok = warp_wait(&p_full[t], il & 1, ctl))) break;
-          tc_fence_after();
-          issue_pv(t, stl, true, 1);
+          // unrolled over the compile-time tile count, so every descriptor
+          // offset stays a constant (a runtime trip count here slows the whole
+          // forward by ~8%: the issuing code must never pause)
+#pragma unroll
+          for (int t = 0; t < QT; ++t) {
+            if (t >= qt_n) break;
+            if (i > 0) {
+              // PV of the first 64 keys while the softmax warps store the rest of P
+              if (!(ok = warp_wait(&p_half[t], (i - 1) & 1, ctl))) break;
+              if (t == 0 && !(ok = warp_wait(L::ONES_IN_V ? &v_rdy[stp] : &v_full[stp], php, ctl))) break;
+              tc_fence_after();
+              issue_pv(t, stp, i - 1 > 0, 0);
+              if (!(ok = warp_wait(&p_full[t], (i - 1) & 1, ctl))) break;
+              tc_fence_after();
+              issue_pv(t, stp, true, 1);
+            }
+            issue_qk(t, st);
+            umma_commit(&s_full[t]);
+          }
+          if (!ok) break;
+          umma_commit(&k_empty[st]);
+          if (i > 0) umma_commit(&v_empty[stp]);
         }
         if (ok) {
-          umma_commit(&v_empty[stl]);
-          umma_commit(o_full);
+          const int il = n_local - 1;
+          const int stl = il % NS;
+#pragma unroll
+          for (int t = 0; t < QT; ++t) {
+            if (!ok || t >= qt_n) break;
+            if (!(ok = warp_wait(&p_half[t], il & 1, ctl))) break;
+            if (t == 0 && !(ok = warp_wait(L::ONES_IN_V ? &v_rdy[stl] : &v_full[stl], (il / NS) & 1, ctl)))
+              break;
+            tc_fence_after();
+            issue_pv(t, stl, il > 0, 0);
+            if (!(ok = warp_wait(&p_full[t], il & 1, ctl))) break;
+            tc_fence_after();
+            issue_pv(t, stl, true, 1);
+          }
+          if (ok) {
+            umma_commit(&v_empty[stl]);
+            umma_commit(o_full);
+          }
         }
       }
     }
-  } else if (ROPE && (warp == 10 || warp == 11) && n_local > 0) {
+  } else if (ROPE && n_local > 0) {
     // ------------------------------------------------------------ RoPE re-shift of the sink
     // Queries, in-flight keys and ring keys carry their temporal rotation at
     // stream positions.  Re-shifting (Sec. 3.5) moves the window back by the
@@ -430,9 +517,10 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
     // rope_shift frames does.  That happens here, in shared memory, between
     // the TMA copy of a sink tile and the MMAs that read it: channel pair
     // (2i, 2i+1), i < rope_dims / 2, turns by rope_shift * base^(-2i/rope_dims).
-    // Each of the two warps turns its own half of every sink tile (rows
+    // With two helper warps each turns its own half of every sink tile (rows
     // [64 h, 64 h + 64)), so they never wait for each other.
-    const int half = warp - 10;
+    const int half = warp - 9 - L::ISSUERS;
+    constexpr int kRows = kTileRows / L::HELPERS;  // of a helper
     float2* cs = reinterpret_cast<float2*>(smem + L::OFF_ROPE + half * L::ROPE_WARP_BYTES);
     const int pairs = p.rope_dims / 2;
     for (int i = lane; i < pairs; i += 32) cs[i] = rope_cos_sin(p.rope_shift, rope_om.hi[i], rope_om.lo[i]);
@@ -453,8 +541,8 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       const int st = i % NS;
       if (!warp_wait(&k_full[st], (i / NS) & 1, ctl)) break;
       const TileSrc src = tile_src(g, j0 + i);
-      const int r_lo = 64 * half;
-      const int nrows = min(64, src.end - src.row0 - r_lo);  // valid rows of this half
+      const int r_lo = kRows * half;
+      const int nrows = min(kRows, src.end - src.row0 - r_lo);  // valid rows of this part
       if (active && nrows > 0) {
         uint8_t* tile = sK + st * L::TILE_BYTES + region_off;
 #pragma unroll 2
@@ -474,13 +562,14 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&k_rdy[st]);
     }
-  } else if (L::ONES_IN_V && (warp == 10 || warp == 11) && n_local > 0) {
+  } else if (L::ONES_IN_V && n_local > 0) {
     // ------------------------------------------------------------ ones columns of V
     // columns DM..DM+15 of each V tile hold bf16 ones (the row-sum columns of
     // the PV MMA); TMA zero-fills them on every load, so they are written
     // again after each one: 16-byte chunks (DM-64)/8 and (DM-64)/8 + 1 of
     // region 1's 128-byte rows, at their 128-byte-swizzle positions
-    const int half = warp - 10;
+    constexpr int kRows = kTileRows / L::HELPERS;  // of a helper
+    const int r_lo = kRows * (warp - 9 - L::ISSUERS);
     const int c0 = (DM - 64) / 8;
     const uint4 ones = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
     for (int i = 0; i < n_local; ++i) {
@@ -488,8 +577,8 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       if (!warp_wait(&v_full[st], (i / NS) & 1, ctl)) break;
       uint8_t* reg1 = sV + st * L::TILE_BYTES + L::REGION_BYTES;
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int r = 64 * half + 32 * k + lane;
+      for (int k = 0; k < kRows / 32; ++k) {
+        const int r = r_lo + 32 * k + lane;
         *reinterpret_cast<uint4*>(reg1 + r * 128 + ((c0 ^ (r & 7)) << 4)) = ones;
         *reinterpret_cast<uint4*>(reg1 + r * 128 + (((c0 + 1) ^ (r & 7)) << 4)) = ones;
       }
@@ -521,13 +610,22 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       if (!(ok = warp_wait(&s_full[t], i & 1, ctl))) break;
       tc_fence_after();
       float s[128];
+      if constexpr (L::SPLIT_P) {
+        uint32_t r[4][32];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        uint32_t r[32];
-        tmem_ld32(s_addr + 32 * c, r);
+        for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + 32 * c, r[c]);
         tmem_wait_ld();
 #pragma unroll
-        for (int k = 0; k < 32; ++k) s[32 * c + k] = __uint_as_float(r[k]);
+        for (int c = 0; c < 128; ++c) s[c] = __uint_as_float(r[c / 32][c % 32]);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          uint32_t r[32];
+          tmem_ld32(s_addr + 32 * c, r);
+          tmem_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 32; ++k) s[32 * c + k] = __uint_as_float(r[k]);
+        }
       }
       const int limit = (src.seg != kSegOwn ? src.end : c_limit) - src.row0;
       if (limit < kTileRows) {
@@ -535,6 +633,30 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
         for (int c = 0; c < 128; ++c)
           if (c >= limit) s[c] = -INFINITY;
       }
+      // P of keys 32 g4 + 2 k and + 1, as a bf16 pair, relative to a maximum
+      const float2 sl2x2 = make_float2(sl2, sl2);
+      auto minus = [](float m) {
+        const float m_eff = (m == -INFINITY) ? 0.f : m;
+        return make_float2(-m_eff, -m_eff);
+      };
+      auto weights = [&](int g4, int k, float2 negm) {
+        const float2 x = fma2(make_float2(s[32 * g4 + 2 * k], s[32 * g4 + 2 * k + 1]), sl2x2, negm);
+        return pack_bf16x2(ex2_approx(x.x), ex2_approx(x.y));
+      };
+      // The first groups against the maximum so far, which the tile hardly ever
+      // replaces (they are redone then): their exponentials overlap the loads
+      // and the maximum instead of waiting for them.  A tile's softmax alone
+      // took 1024 cycles without them, 848 with two groups, 875 with three;
+      // where the tiles' softmaxes take turns (d = 128) it gained nothing.
+      constexpr int kEarly = L::SPLIT_P ? 2 : 0;
+      [[maybe_unused]] uint32_t early[kEarly > 0 ? kEarly : 1][16];
+      auto set_early = [&](float2 negm) {
+#pragma unroll
+        for (int g4 = 0; g4 < kEarly; ++g4)
+#pragma unroll
+          for (int k = 0; k < 16; ++k) early[g4][k] = weights(g4, k, negm);
+      };
+      set_early(minus(m_used));
       float mq[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) mq[k] = fmaxf(s[k], s[k + 4]);
@@ -557,8 +679,13 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
           alpha = ex2_approx(m_used - m_cand);
           m_used = m_cand;
         }
+        set_early(minus(m_used));
         l *= alpha;
         if (i > 0) {
+          if constexpr (L::SPLIT_P) {  // (else S of this tile implies it)
+            if (!(ok = warp_wait(&pv_done[t], (i - 1) & 1, ctl))) break;
+            tc_fence_after();
+          }
           // exactly the tile's O columns (the next tile's O follows them)
 #pragma unroll
           for (int c = 0; c < DM / 32; ++c) {
@@ -588,9 +715,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
           tmem_wait_st();
         }
       }
-      const float m_eff = (m_used == -INFINITY) ? 0.f : m_used;
-      const float2 sl2x2 = make_float2(sl2, sl2);
-      const float2 negm = make_float2(-m_eff, -m_eff);
+      const float2 negm = minus(m_used);
       float2 acc = make_float2(0.f, 0.f);
       // P in four 32-key groups, each stored as soon as it is packed; the first
       // two groups (keys 0..63) are announced while the third is stored
@@ -599,8 +724,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
         uint32_t packed[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-          const float2 x = fma2(make_float2(s[32 * g4 + 2 * k], s[32 * g4 + 2 * k + 1]), sl2x2, negm);
-          const uint32_t pk = pack_bf16x2(ex2_approx(x.x), ex2_approx(x.y));
+          const uint32_t pk = g4 < kEarly ? early[g4 < kEarly ? g4 : 0][k] : weights(g4, k, negm);
           // the row sum uses the bf16 weights the PV MMA consumes, so O is an
           // exact convex combination of them (d = 64: summed by the MMA)
           if constexpr (!L::SUM_MMA)
@@ -612,9 +736,16 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&p_half[t]);
+          // the previous tile's PV has read the columns of the second half
+          if (L::SPLIT_P && i > 0) {
+            if (!(ok = warp_wait(&pv_done[t], (i - 1) & 1, ctl))) break;
+            tc_fence_after();
+          }
         }
-        tmem_st16(s_addr + 16 * g4, packed);
+        const uint32_t p_addr = L::SPLIT_P && g4 >= 2 ? lane_base + L::P_COL(t, 1) : s_addr + 32 * (g4 >> 1);
+        tmem_st16(p_addr + 16 * (g4 & 1), packed);
       }
+      if (!ok) break;
       l += acc.x + acc.y;
       tmem_wait_st();
       tc_fence_before();
@@ -828,7 +959,7 @@ cudaError_t launch_fwd_t(const CUtensorMap& tq, const CUtensorMap& tk, const CUt
                          const CUtensorMap& tkr, const CUtensorMap& tvr, const CUtensorMap& tks,
                          const CUtensorMap& tvs, const CUtensorMap& top, const FwdParams& p,
                          const RopeFreq& om, cudaStream_t s) {
-  using L = FwdLayout<D, DM, ROPE>;
+  using L = FwdLayout<D, DM, ROPE, SPLIT>;
   static bool attr_set = false;  // per process; the attribute is per function
   if (!attr_set) {
     // The in-kernel register re-split assumes the launch register count; with

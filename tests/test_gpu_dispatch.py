@@ -59,3 +59,23 @@ def test_output_rows_at_16_and_32_bytes(mw, d):
         assert torch.equal(a, b)
     o_ref, _ = oracle.fwd(q.cpu(), k.cpu(), v.cpu(), T, d ** -0.5)
     assert float((results[0][0].double().cpu() - o_ref).norm() / o_ref.norm()) <= 5e-3
+
+
+@pytest.mark.parametrize("rise", [8.0, 0.0, -8.0])  # of the scores, from a 128-key tile to the next
+@pytest.mark.parametrize("d", [64, 72, 80])
+@pytest.mark.parametrize("T,n", [(1, 1), (64, 1), (128, 1), (129, 1), (257, 1), (100, 5), (300, 3)])
+def test_weights_in_columns_of_their_own(mw, T, n, d, rise):
+    """Up to 80 channels a tile's weights are split over two column ranges and
+    begun with the maximum of the tiles before it: maxima that grow by more
+    than 2^8 in each tile (all weights redone, O rescaled), that hardly move,
+    and that fall, over one to eight key tiles.  The weights and O are rounded
+    to bf16 (2^-9 each): 5e-3 of O's norm, 2^-8 of the row sum."""
+    g = torch.Generator().manual_seed(d * 1000 + T * 7 + n)
+    N = n * T
+    q, k, v = (torch.randn(1, 3, N, d, generator=g).to(torch.bfloat16) for _ in range(3))
+    q[..., 0] = d ** 0.5
+    k[..., 0] = rise * (torch.arange(N) // 128)
+    o, lse = mw.mw_bca_fwd(q.cuda(), k.cuda(), v.cuda(), T)
+    o_ref, lse_ref = oracle.fwd(q, k, v, T, d ** -0.5)
+    assert float((o.cpu().double() - o_ref).norm() / o_ref.norm()) <= 5e-3
+    assert float((lse.cpu().double() - lse_ref).abs().max()) <= 2.0 ** -8
