@@ -96,9 +96,9 @@ struct BwdLayout {
   static constexpr int OFF_ONES = OFF_DELTA + 2 * VEC_BYTES;
   static constexpr int OFF_BAR = OFF_ONES + ONES_BYTES;
   // kv_full, q_full, q_empty [QSTAGES], do_full, do_empty [DOSTAGES], s_full,
-  // s_free, dp_full, dp_free, pt_ready, pt_free, p_ready, dq_full, dq_free,
+  // s_free, dp_full, dp_free, pt_ready, p_ready, dq_full, dq_free,
   // ds_free[DS_BUFS], dkv_full
-  static constexpr int NBAR = 1 + 2 * (QSTAGES + DOSTAGES) + 10 + DS_BUFS;
+  static constexpr int NBAR = 1 + 2 * (QSTAGES + DOSTAGES) + 9 + DS_BUFS;
   static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
   static constexpr int BYTES = OFF_MISC + 16;
   // d = 128 has no room for separate S^T, dP^T, P^T and dQ^T columns: P^T
@@ -198,8 +198,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
   uint64_t* dp_full = s_free + 1;
   uint64_t* dp_free = dp_full + 1;
   uint64_t* pt_ready = dp_free + 1;
-  uint64_t* pt_free = pt_ready + 1;
-  uint64_t* p_ready = pt_free + 1;
+  uint64_t* p_ready = pt_ready + 1;
   uint64_t* dq_full = p_ready + 1;
   uint64_t* dq_free = dq_full + 1;
   uint64_t* ds_free = dq_free + 1;
@@ -264,7 +263,6 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
     mbar_init(dp_full, 1);
     mbar_init(dp_free, 8);
     mbar_init(pt_ready, 8);
-    mbar_init(pt_free, 1);
     mbar_init(p_ready, 8);
     mbar_init(dq_full, 1);
     mbar_init(dq_free, 4);
@@ -491,7 +489,6 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
             tc_fence_after();
             issue_dv(j);
             umma_commit(&do_empty[j % ND]);
-            umma_commit(pt_free);
             if (more) {
               // dP^T of the next step once the P/dS warps hold dP^T_j
               if (!(ok = warp_wait(dp_free, j & 1, ctl))) break;
@@ -596,11 +593,13 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       }
       // P^T (bf16 pairs) -> TMEM right away, so that dV_j starts while dS_j is
       // computed
+      uint32_t r[32];  // 32 columns of dP^T
       if constexpr (!L::PAIRED) {
-        if (j > 0) {  // dV_{j-1} has read P^T_{j-1}
-          if (!(ok = warp_wait(pt_free, (j - 1) & 1, ctl))) break;
-          tc_fence_after();
-        }
+        // dP^T_j is issued after dV_{j-1}: once it is there, dV_{j-1} has read
+        // P^T_{j-1}.  Its first half loads while P^T is stored.
+        if (!(ok = warp_wait(dp_full, j & 1, ctl))) break;
+        tc_fence_after();
+        tmem_ld32(dp_addr, r);
       }
       {
         uint32_t pe[CW / 2];
@@ -612,13 +611,22 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(pt_ready);
       }
-      if (!(ok = warp_wait(dp_full, j & 1, ctl))) break;
-      tc_fence_after();
+      if constexpr (L::PAIRED) {
+        if (!(ok = warp_wait(dp_full, j & 1, ctl))) break;
+        tc_fence_after();
+        tmem_ld32(dp_addr, r);
+      }
+      // the wait for the dS^T buffer passes while dP^T loads, not in the
+      // serial chain of the step that these warps are (16 heads of 72
+      // channels, 16 x 880: 1309 -> 1295 us)
+      const int buf = j % L::DS_BUFS;
+      if (j >= L::DS_BUFS &&
+          !(ok = warp_wait(&ds_free[buf], ((j / L::DS_BUFS) - 1) & 1, ctl)))
+        break;
       uint32_t dk[CW / 2];
 #pragma unroll
       for (int h = 0; h < CW / 32; ++h) {
-        uint32_t r[32];
-        tmem_ld32(dp_addr + 32 * h, r);
+        if (h > 0) tmem_ld32(dp_addr + 32 * h, r);
         tmem_wait_ld();
         if (!L::PAIRED && h == CW / 32 - 1) {
           // dP^T is in registers: its columns can take the next step's dP^T
@@ -644,10 +652,6 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         }
       }
       // dS^T row segment -> shared memory (swizzled like a TMA 128-byte tile)
-      const int buf = j % L::DS_BUFS;
-      if (j >= L::DS_BUFS &&
-          !(ok = warp_wait(&ds_free[buf], ((j / L::DS_BUFS) - 1) & 1, ctl)))
-        break;
       uint8_t* ds_row = sDS + buf * L::DS_BYTES + ds_off;
 #pragma unroll
       for (int q = 0; q < CW / 8; ++q)
