@@ -79,3 +79,26 @@ def test_weights_in_columns_of_their_own(mw, T, n, d, rise):
     o_ref, lse_ref = oracle.fwd(q, k, v, T, d ** -0.5)
     assert float((o.cpu().double() - o_ref).norm() / o_ref.norm()) <= 5e-3
     assert float((lse.cpu().double() - lse_ref).abs().max()) <= 2.0 ** -8
+
+
+@pytest.mark.parametrize("d,rope", [(64, 64), (64, 6), (72, 24), (80, 80), (128, 32)])
+@pytest.mark.parametrize("W,T,length,sink", [(1, 64, 0, 32), (1, 128, 300, 130), (2, 100, 640, 300), (3, 200, 512, 16)])
+def test_turned_sink_without_a_split(mw, W, T, length, sink, d, rope):
+    """The sink's key tiles turned by one helper warp (d = 64: its sibling
+    issues MMAs) or by two, key range in one piece, one query tile or more:
+    the tolerances of the split form's parity."""
+    g = torch.Generator().manual_seed(d * 10 + W + sink)
+    cap, head, shift, sc = 640, 100, 12, d ** -0.5
+    q, kn, vn = (torch.randn(1, 2, W * T, d, generator=g).to(torch.bfloat16) for _ in range(3))
+    kr, vr = (torch.randn(1, 2, cap, d, generator=g).to(torch.bfloat16) for _ in range(2))
+    ks, vs = (torch.randn(1, 2, sink, d, generator=g).to(torch.bfloat16) for _ in range(2))
+    mw.mw_set_option("cache_splits", 1)
+    try:
+        o, lse = mw.mw_bca_cache_fwd_rope(q.cuda(), kn.cuda(), vn.cuda(), ks.cuda(), vs.cuda(), kr.cuda(),
+                                          vr.cuda(), head, length, T, rope, 1e4, shift, sc)
+    finally:
+        mw.mw_set_option("cache_splits", 0)
+    o_ref, lse_ref = oracle.cache_fwd_reshift(q, kn, vn, kr, vr, cap, head, length, T, sc, ks, vs, rope, 1e4, shift)
+    o, lse = o.cpu().double(), lse.cpu().double()
+    assert float((o - o_ref).norm() / o_ref.norm()) <= 5e-3 and float((o - o_ref).abs().max()) <= 2e-2
+    assert bool(((lse - lse_ref).abs() <= 1e-3 * lse_ref.abs().clamp(min=1)).all())
