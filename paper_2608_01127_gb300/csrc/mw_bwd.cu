@@ -96,9 +96,12 @@ struct BwdLayout {
   static constexpr int OFF_ONES = OFF_DELTA + 2 * VEC_BYTES;
   static constexpr int OFF_BAR = OFF_ONES + ONES_BYTES;
   // kv_full, q_full, q_empty [QSTAGES], do_full, do_empty [DOSTAGES], s_full,
-  // s_free, dp_full, dp_free, pt_ready, p_ready, dq_full, dq_free,
-  // ds_free[DS_BUFS], dkv_full
-  static constexpr int NBAR = 1 + 2 * (QSTAGES + DOSTAGES) + 9 + DS_BUFS;
+  // s_free, dp_full, dp_free, pt_ready, p_ready[DS_BUFS], dq_full, dq_free,
+  // ds_free[DS_BUFS], dkv_full.  p_ready is one per dS^T buffer, as ds_free is:
+  // the P/dS warps run up to a buffer ahead of the issuer of dQ and dK, and a
+  // single barrier could complete its next phase before that warp has looked at
+  // this one; its parity would then never match again.
+  static constexpr int NBAR = 1 + 2 * (QSTAGES + DOSTAGES) + 8 + 2 * DS_BUFS;
   static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
   static constexpr int BYTES = OFF_MISC + 16;
   // d = 128 has no room for separate S^T, dP^T, P^T and dQ^T columns: P^T
@@ -199,7 +202,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
   uint64_t* dp_free = dp_full + 1;
   uint64_t* pt_ready = dp_free + 1;
   uint64_t* p_ready = pt_ready + 1;
-  uint64_t* dq_full = p_ready + 1;
+  uint64_t* dq_full = p_ready + L::DS_BUFS;
   uint64_t* dq_free = dq_full + 1;
   uint64_t* ds_free = dq_free + 1;
   uint64_t* dkv_full = ds_free + L::DS_BUFS;
@@ -263,10 +266,12 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
     mbar_init(dp_full, 1);
     mbar_init(dp_free, 8);
     mbar_init(pt_ready, 8);
-    mbar_init(p_ready, 8);
     mbar_init(dq_full, 1);
     mbar_init(dq_free, 4);
-    for (int b = 0; b < L::DS_BUFS; ++b) mbar_init(&ds_free[b], 1);
+    for (int b = 0; b < L::DS_BUFS; ++b) {
+      mbar_init(&p_ready[b], 8);
+      mbar_init(&ds_free[b], 1);
+    }
     mbar_init(dkv_full, 2);
     *abort_flag = 0;
     fence_mbar_init();
@@ -445,7 +450,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
         } else {
           for (int j = 0; ok && j < n_q; ++j) {
             // dS_j is in shared memory (and so dP_j in registers)
-            if (!(ok = warp_wait(p_ready, j & 1, ctl))) break;
+            if (!(ok = warp_wait(&p_ready[j % L::DS_BUFS], (j / L::DS_BUFS) & 1, ctl))) break;
             tc_fence_after();
             issue_dq(j);
             umma_commit(dq_full);
@@ -500,7 +505,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
             }
           }
           if (!role_a) {
-            if (!(ok = warp_wait(p_ready, j & 1, ctl))) break;
+            if (!(ok = warp_wait(&p_ready[j % L::DS_BUFS], (j / L::DS_BUFS) & 1, ctl))) break;
             tc_fence_after();
             // dQ_j first, so the drain starts while dK_j runs
             if (j > 0) {
@@ -660,7 +665,7 @@ __global__ void __launch_bounds__(BwdLayout<D, DM>::THREADS, 1)
       fence_proxy_async_smem();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_ready);
+      if (lane == 0) mbar_arrive(&p_ready[buf]);
     }
     // ---- epilogue: warpgroup 0 writes dK (x scale), warpgroup 1 writes dV
     // (zeros if a wait gave up: the rows get a defined value either way)
