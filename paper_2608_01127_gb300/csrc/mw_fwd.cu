@@ -850,20 +850,18 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
 }
 
 // Merge of split-KV partials (per row): LSE = ln sum_s exp(LSE_s),
-// O = sum_s exp(LSE_s - LSE) O_s.  D / 8 lanes per row, 8 columns each, and
-// kCombineRows rows a lane, all of whose loads are issued before the first is
-// used (S splits, 2 to 4; S = 0: any number, one after another): the partials
-// come from L2, so bytes in flight bound it (a warp a row with one 16-byte load
-// a split: streaming step of 12 heads of 64, three splits, 15.9 us a step, this
-// form 14.3; 16 heads of 128, 4 x 880 rows, two splits, combine alone 17.4 ->
-// 15.6 us).  The blocks after those carry the
-// ring commit cj (one thread per 16-byte piece of a committed row of one
-// head), when there is one.
-constexpr int kCombineRows = 2;
-template <int D>
-constexpr int combine_block_rows() {
-  return kCombineRows * 256 / (D / 8);
-}
+// O = sum_s exp(LSE_s - LSE) O_s.  D / 8 lanes per row, 8 columns each: the
+// partials come from L2, so bytes in flight bound it, and a launch has few rows
+// (more splits, fewer rows), so a lane takes one row and issues all its loads
+// before it uses the first (S splits, 2 to 8; S = 0: any number, eight at a
+// time).  A step (forward and combine), us, with two rows a lane and one split
+// after another from five splits on -> this form: 8 heads of 64, 200 new rows,
+// five splits against one chunk 11.1 -> 7.6, eleven against twelve chunks 15.6
+// -> 9.8; 12 of 128, 440 rows, five splits 16.1 -> 13.2; 12 of 128, 880 rows,
+// three splits 17.9 -> 17.7; 16 of 128, 880 rows, two splits 20.9 -> 20.5.  (A
+// warp a row with one 16-byte load a split: 8.7, 11.6, 14.5, 19.4 and 20.7.)
+// The blocks after those of the rows carry the ring commit cj (one thread per
+// 16-byte piece of a committed row of one head), when there is one.
 template <int D, int S>
 __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ o_part,
                                                       const float* __restrict__ lse_part,
@@ -874,7 +872,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
   pdl_wait();     // the forward's partials (and its reads of the ring) are complete
   pdl_trigger();  // the next step's forward may start its setup meanwhile
   constexpr int G = D / 8;  // lanes per row
-  constexpr int kBlockRows = combine_block_rows<D>();
+  constexpr int kBlockRows = 256 / G;
   const int combine_blocks = (n_rows + kBlockRows - 1) / kBlockRows;
   if (static_cast<int>(blockIdx.x) >= combine_blocks) {
     const long long idx =
@@ -886,72 +884,63 @@ __global__ void __launch_bounds__(256) combine_kernel(const float* __restrict__ 
   }
   const int d_io = (D == 64) ? D : d_io_arg;  // padded head dims use the 128-wide kernels
   const int sub = threadIdx.x % G;
+  const int row = blockIdx.x * kBlockRows + threadIdx.x / G;
   // (the multiples of 8 columns past the caller's hold nothing)
   if (8 * sub >= d_io) return;
-  const int row0 = blockIdx.x * kBlockRows + threadIdx.x / G;
-  constexpr int kStep = 256 / G;  // rows between a lane's rows
-  constexpr int NS = S > 0 ? S : 1;
+  constexpr int kAll = S > 0 ? S : kMaxSplits;
+  constexpr int kChunk = S > 0 ? S : 8;  // splits whose columns are in registers at once
+  const int n = S > 0 ? S : splits;
   const size_t split_stride = static_cast<size_t>(n_rows) * D;
-  float ls[kCombineRows][NS];
-  float4 x[kCombineRows][NS][2];
-  auto load = [&](int r, int k, int s) {
-    const int row = row0 + r * kStep;
-    const float4* src =
-        reinterpret_cast<const float4*>(o_part + s * split_stride + static_cast<size_t>(row) * D) + 2 * sub;
-    x[r][k][0] = src[0];
-    x[r][k][1] = src[1];
-  };
-  if constexpr (S > 0) {
+  float ls[kAll], acc[8], m = -INFINITY, wsum = 0.f;
+  float4 x[kChunk][2];
 #pragma unroll
-    for (int r = 0; r < kCombineRows; ++r)
+  for (int k = 0; k < 8; ++k) acc[k] = 0.f;
 #pragma unroll
-      for (int s = 0; s < S; ++s)
-        if (row0 + r * kStep < n_rows) {
-          ls[r][s] = lse_part[static_cast<size_t>(s) * n_rows + row0 + r * kStep];
-          load(r, s, s);
-        }
-  }
+  for (int s = 0; s < kAll; ++s)
+    if (s < n && row < n_rows) ls[s] = lse_part[static_cast<size_t>(s) * n_rows + row];
 #pragma unroll
-  for (int r = 0; r < kCombineRows; ++r) {
-    const int row = row0 + r * kStep;
-    if (row >= n_rows) return;
-    float acc[8];
+  for (int s0 = 0; s0 < kAll; s0 += kChunk) {
+    if (s0 >= n) break;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = 0.f;
-    float wsum = 0.f, m = -INFINITY;
+    for (int k = 0; k < kChunk; ++k)
+      if (s0 + k < n && row < n_rows) {
+        const float4* src = reinterpret_cast<const float4*>(
+            o_part + (s0 + k) * split_stride + static_cast<size_t>(row) * D + 8 * sub);
+        x[k][0] = src[0];
+        x[k][1] = src[1];
+      }
+    // (tested again here, and not left early above: with both parts in one
+    // block the compiler moves each load next to its use)
+    if (row >= n_rows) break;
+    if (s0 == 0) {
+#pragma unroll
+      for (int s = 0; s < kAll; ++s)
+        if (s < n) m = fmaxf(m, ls[s]);
+    }
     // a split whose LSE is -inf saw no key of the row: its O part is skipped
     // (never multiplied: it may hold anything)
-    auto add = [&](float l, const float4 (&v)[2]) {
-      const float w = l == -INFINITY ? 0.f : __expf(l - m);
+#pragma unroll
+    for (int k = 0; k < kChunk; ++k) {
+      if (s0 + k >= n) break;
+      const float w = ls[s0 + k] == -INFINITY ? 0.f : __expf(ls[s0 + k] - m);
       wsum += w;
       if (w > 0.f) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          acc[4 * h] += w * v[h].x;
-          acc[4 * h + 1] += w * v[h].y;
-          acc[4 * h + 2] += w * v[h].z;
-          acc[4 * h + 3] += w * v[h].w;
+          acc[4 * h] += w * x[k][h].x;
+          acc[4 * h + 1] += w * x[k][h].y;
+          acc[4 * h + 2] += w * x[k][h].z;
+          acc[4 * h + 3] += w * x[k][h].w;
         }
       }
-    };
-    if constexpr (S > 0) {
-#pragma unroll
-      for (int s = 0; s < S; ++s) m = fmaxf(m, ls[r][s]);
-#pragma unroll
-      for (int s = 0; s < S; ++s) add(ls[r][s], x[r][s]);
-    } else {
-      for (int s = 0; s < splits; ++s) m = fmaxf(m, lse_part[static_cast<size_t>(s) * n_rows + row]);
-      for (int s = 0; s < splits; ++s) {
-        load(r, 0, s);
-        add(lse_part[static_cast<size_t>(s) * n_rows + row], x[r][0]);
-      }
     }
-    const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
-    *reinterpret_cast<uint4*>(o + static_cast<size_t>(row) * d_io + 8 * sub) =
-        make_uint4(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv),
-                   pack_bf16x2(acc[4] * inv, acc[5] * inv), pack_bf16x2(acc[6] * inv, acc[7] * inv));
-    if (lse && sub == 0) lse[row] = wsum > 0.f ? m + __logf(wsum) : -INFINITY;
   }
+  if (row >= n_rows) return;
+  const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
+  *reinterpret_cast<uint4*>(o + static_cast<size_t>(row) * d_io + 8 * sub) =
+      make_uint4(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv),
+                 pack_bf16x2(acc[4] * inv, acc[5] * inv), pack_bf16x2(acc[6] * inv, acc[7] * inv));
+  if (lse && sub == 0) lse[row] = wsum > 0.f ? m + __logf(wsum) : -INFINITY;
 }
 
 template <int D, int DM, bool ROPE, bool SPLIT>
@@ -1011,7 +1000,7 @@ cudaError_t launch_combine(int d, int d_io, const float* o_part, const float* ls
                            const CommitJob& cj, cudaStream_t s) {
   const int n_rows = BH * rows;
   const long long commit_pieces = static_cast<long long>(cj.rows) * (cj.d / 8) * cj.BH;
-  const int block_rows = d == 64 ? combine_block_rows<64>() : combine_block_rows<128>();
+  const int block_rows = 256 / (d / 8);
   const long long blocks = (n_rows + block_rows - 1) / block_rows + (commit_pieces + 255) / 256;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;
@@ -1019,15 +1008,20 @@ cudaError_t launch_combine(int d, int d_io, const float* o_part, const float* ls
   auto launch = [&](auto kernel) {
     return cudaLaunchKernelEx(&cfg, kernel, o_part, lse_part, o, lse, splits, n_rows, d_io, cj);
   };
-  if (d == 64)
-    return launch(splits == 2   ? combine_kernel<64, 2>
-                  : splits == 3 ? combine_kernel<64, 3>
-                  : splits == 4 ? combine_kernel<64, 4>
-                                : combine_kernel<64, 0>);
-  return launch(splits == 2   ? combine_kernel<128, 2>
-                : splits == 3 ? combine_kernel<128, 3>
-                : splits == 4 ? combine_kernel<128, 4>
-                              : combine_kernel<128, 0>);
+  auto by_splits = [&](auto width) {
+    constexpr int D = decltype(width)::value;
+    switch (splits) {
+      case 2: return launch(combine_kernel<D, 2>);
+      case 3: return launch(combine_kernel<D, 3>);
+      case 4: return launch(combine_kernel<D, 4>);
+      case 5: return launch(combine_kernel<D, 5>);
+      case 6: return launch(combine_kernel<D, 6>);
+      case 7: return launch(combine_kernel<D, 7>);
+      case 8: return launch(combine_kernel<D, 8>);
+      default: return launch(combine_kernel<D, 0>);
+    }
+  };
+  return d == 64 ? by_splits(std::integral_constant<int, 64>{}) : by_splits(std::integral_constant<int, 128>{});
 }
 
 }  // namespace mw
