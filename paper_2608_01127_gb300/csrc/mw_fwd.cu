@@ -789,21 +789,11 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       for (int k = 0; k < 32; ++k) v[k] = nonzero ? __uint_as_float(r[k]) * inv_l : 0.f;
       if constexpr (!SPLIT) {
         if (!row_valid) continue;
-        if (p.num_splits == 1) {
-          // the caller's rows hold d_io <= D columns (multiples of 8); only
-          // the 128-wide kernel serves padded head dims
-          const int d_io = (D == 64) ? D : p.d_io;
-          if (32 * c >= d_io) continue;
-          store_row32(p.o + row_off * d_io + 32 * c, v, min(4, (d_io - 32 * c) / 8), p.wide_out);
-        } else {
-          // never taken (the launcher picks SPLIT for several splits), but
-          // with this row-per-thread form of the partials here the compiler
-          // schedules the training kernel 1.4% faster at d = 128
-          float4* dst = reinterpret_cast<float4*>(
-              p.o_part + (static_cast<size_t>(split) * p.BH * p.rows_q + row_off) * D + 32 * c);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) dst[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-        }
+        // the caller's rows hold d_io <= D columns (multiples of 8); only
+        // the 128-wide kernel serves padded head dims
+        const int d_io = (D == 64) ? D : p.d_io;
+        if (32 * c >= d_io) continue;
+        store_row32(p.o + row_off * d_io + 32 * c, v, min(4, (d_io - 32 * c) / 8), p.wide_out);
       } else if (t < qt_n) {
         // (an empty tile's warps skip the O wait: they must not touch the
         // stages, which the other tile's MMAs may still be reading)
@@ -832,7 +822,7 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       }
     }
     if (row_valid) {
-      if (!SPLIT && p.num_splits == 1) {
+      if constexpr (!SPLIT) {
         if (p.lse) p.lse[row_off] = lse;
       } else {
         p.lse_part[static_cast<size_t>(split) * p.BH * p.rows_q + row_off] = lse;
