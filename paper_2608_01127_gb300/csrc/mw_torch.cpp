@@ -142,13 +142,24 @@ PyObject* result(std::initializer_list<const at::Tensor*> ts) {
   return tup;
 }
 
+// Runs f without the interpreter lock (a launch can wait for room in the
+// stream's queue).  A guard, since f may throw: a data pointer of a lazily
+// cloned tensor is a copy, which can run out of memory.
+class WithoutLock {
+ public:
+  WithoutLock() : state_(PyEval_SaveThread()) {}
+  ~WithoutLock() { PyEval_RestoreThread(state_); }
+  WithoutLock(const WithoutLock&) = delete;
+  WithoutLock& operator=(const WithoutLock&) = delete;
+
+ private:
+  PyThreadState* state_;
+};
+
 template <class F>
 mw_status call(F&& f) {
-  // (a launch can wait for room in the stream's queue)
-  PyThreadState* st = PyEval_SaveThread();
-  const mw_status s = f();
-  PyEval_RestoreThread(st);
-  return s;
+  WithoutLock unlocked;
+  return f();
 }
 
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
