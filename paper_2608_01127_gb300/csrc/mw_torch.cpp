@@ -24,6 +24,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <array>
 #include <climits>
 #include <cmath>
 #include <initializer_list>
@@ -121,8 +122,16 @@ Span span(const at::Tensor& t) {
   return {p, p + t.nbytes()};
 }
 
-at::Tensor rows_f32(const at::Tensor& q) {
-  return at::empty({q.size(0), q.size(1), q.size(2)}, q.options().dtype(at::kFloat));
+// Sizes of a [B, H, rows, d] tensor, as the outputs are allocated from them.
+using Shape = std::array<int64_t, 4>;
+Shape shape(const at::Tensor& t) { return {t.size(0), t.size(1), t.size(2), t.size(3)}; }
+
+at::Tensor rows_f32(const Shape& s, const at::TensorOptions& options) {
+  return at::empty({s[0], s[1], s[2]}, options.dtype(at::kFloat));
+}
+
+at::Tensor scratch(size_t bytes, const at::TensorOptions& options) {
+  return at::empty({static_cast<int64_t>(bytes)}, options.dtype(at::kByte));
 }
 
 PyObject* none() { Py_RETURN_NONE; }
@@ -142,9 +151,12 @@ PyObject* result(std::initializer_list<const at::Tensor*> ts) {
   return tup;
 }
 
-// Runs f without the interpreter lock (a launch can wait for room in the
-// stream's queue).  A guard, since f may throw: a data pointer of a lazily
-// cloned tensor is a copy, which can run out of memory.
+// Runs f, which allocates the outputs and launches, without the interpreter lock:
+// an allocation can wait for the device, a launch for room in the stream's queue,
+// and what they wait for can be a callback that needs the lock.  Sizes and data
+// pointers of the arguments are taken before, with the lock.  A guard, since f
+// may throw (out of memory).  f returns false for outputs that are not real
+// tensors (is_real), and sets the status otherwise.
 class WithoutLock {
  public:
   WithoutLock() : state_(PyEval_SaveThread()) {}
@@ -157,7 +169,7 @@ class WithoutLock {
 };
 
 template <class F>
-mw_status call(F&& f) {
+auto call(F&& f) {
   WithoutLock unlocked;
   return f();
 }
@@ -197,17 +209,23 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
       !one_device({q, k, v}, &dev) || !small_int(a[3], &T) || T < 1 || q->size(2) % T ||
       !softmax_scale(a[4], q->size(3), &scale) || !PyBool_Check(a[5]))
     return none();
-  at::Tensor o = at::empty(q->sizes(), q->options());
-  at::Tensor lse = a[5] == Py_True ? rows_f32(*q) : at::Tensor();
-  if (!is_real(o) || (lse.defined() && !is_real(lse))) return none();
-  const mw_status s = call([&] {
-    return p_fwd(q->const_data_ptr(), k->const_data_ptr(), v->const_data_ptr(),
-                 o.mutable_data_ptr(),
-                 lse.defined() ? static_cast<float*>(lse.mutable_data_ptr()) : nullptr,
-                 static_cast<int>(q->size(0)), static_cast<int>(q->size(1)),
-                 static_cast<int>(q->size(2) / T), T, static_cast<int>(q->size(3)), scale,
-                 c10::cuda::getCurrentCUDAStream(dev).stream());
+  const Shape sh = shape(*q);
+  const at::TensorOptions options = q->options();
+  const void *pq = q->const_data_ptr(), *pk = k->const_data_ptr(), *pv = v->const_data_ptr();
+  const bool need_lse = a[5] == Py_True;
+  at::Tensor o, lse;
+  mw_status s = MW_OK;
+  const bool real = call([&] {
+    o = at::empty(sh, options);
+    if (need_lse) lse = rows_f32(sh, options);
+    if (!is_real(o) || (need_lse && !is_real(lse))) return false;
+    s = p_fwd(pq, pk, pv, o.mutable_data_ptr(),
+              need_lse ? static_cast<float*>(lse.mutable_data_ptr()) : nullptr,
+              static_cast<int>(sh[0]), static_cast<int>(sh[1]), static_cast<int>(sh[2] / T), T,
+              static_cast<int>(sh[3]), scale, c10::cuda::getCurrentCUDAStream(dev).stream());
+    return true;
   });
+  if (!real) return none();
   if (s != MW_OK) return PyLong_FromLong(s);
   return result({&o, &lse});
   END_HANDLE_TH_ERRORS
@@ -228,21 +246,28 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
       !one_device({q, k, v, o, lse, dout}, &dev) || !small_int(a[6], &T) || T < 1 ||
       q->size(2) % T || !softmax_scale(a[7], q->size(3), &scale))
     return none();
-  const int B = static_cast<int>(q->size(0)), H = static_cast<int>(q->size(1));
-  const int nc = static_cast<int>(q->size(2) / T), d = static_cast<int>(q->size(3));
+  const Shape sh = shape(*q);
+  const at::TensorOptions options = q->options();
+  const int B = static_cast<int>(sh[0]), H = static_cast<int>(sh[1]);
+  const int nc = static_cast<int>(sh[2] / T), d = static_cast<int>(sh[3]);
   const size_t bytes = p_bwd_ws(B, H, nc, T, d);
-  at::Tensor ws = at::empty({static_cast<int64_t>(bytes)}, q->options().dtype(at::kByte));
-  at::Tensor dq = at::empty(q->sizes(), q->options());
-  at::Tensor dk = at::empty(q->sizes(), q->options());
-  at::Tensor dv = at::empty(q->sizes(), q->options());
-  if (!is_real(ws) || !is_real(dq) || !is_real(dk) || !is_real(dv)) return none();
-  const mw_status s = call([&] {
-    return p_bwd(q->const_data_ptr(), k->const_data_ptr(), v->const_data_ptr(),
-                 o->const_data_ptr(), static_cast<const float*>(lse->const_data_ptr()),
-                 dout->const_data_ptr(), dq.mutable_data_ptr(), dk.mutable_data_ptr(),
-                 dv.mutable_data_ptr(), bytes ? ws.mutable_data_ptr() : nullptr, bytes, B, H, nc,
-                 T, d, scale, c10::cuda::getCurrentCUDAStream(dev).stream());
+  const void *pq = q->const_data_ptr(), *pk = k->const_data_ptr(), *pv = v->const_data_ptr();
+  const void *po = o->const_data_ptr(), *pdo = dout->const_data_ptr();
+  const float* pl = static_cast<const float*>(lse->const_data_ptr());
+  at::Tensor ws, dq, dk, dv;
+  mw_status s = MW_OK;
+  const bool real = call([&] {
+    ws = scratch(bytes, options);
+    dq = at::empty(sh, options);
+    dk = at::empty(sh, options);
+    dv = at::empty(sh, options);
+    if (!is_real(ws) || !is_real(dq) || !is_real(dk) || !is_real(dv)) return false;
+    s = p_bwd(pq, pk, pv, po, pl, pdo, dq.mutable_data_ptr(), dk.mutable_data_ptr(),
+              dv.mutable_data_ptr(), bytes ? ws.mutable_data_ptr() : nullptr, bytes, B, H, nc, T, d,
+              scale, c10::cuda::getCurrentCUDAStream(dev).stream());
+    return true;
   });
+  if (!real) return none();
   if (s != MW_OK) return PyLong_FromLong(s);
   return result({&dq, &dk, &dv});
   END_HANDLE_TH_ERRORS
@@ -290,14 +315,11 @@ PyObject* cache(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const int sink_len = ks ? static_cast<int>(ks->size(2)) : 0;
   const int64_t keys = static_cast<int64_t>(sink_len) + len;
   if (keys > INT_MAX || keys < 0) return none();
-  const int B = static_cast<int>(q->size(0)), H = static_cast<int>(q->size(1));
-  const int W = static_cast<int>(q->size(2) / T), d = static_cast<int>(q->size(3));
+  const Shape sh = shape(*q);
+  const at::TensorOptions options = q->options();
+  const int B = static_cast<int>(sh[0]), H = static_cast<int>(sh[1]);
+  const int W = static_cast<int>(sh[2] / T), d = static_cast<int>(sh[3]);
   const size_t bytes = p_cache_ws(B, H, W, T, d, static_cast<int>(keys));
-  at::Tensor ws;
-  if (bytes > 0 && given && given->nbytes() >= bytes)
-    ws = *given;
-  else if (bytes > 0)
-    ws = at::empty({static_cast<int64_t>(bytes)}, q->options().dtype(at::kByte));
   // what the call writes shares no byte with anything else of the caller's
   Span spans[8];
   int n_spans = 0, n_written = 0;
@@ -310,24 +332,34 @@ PyObject* cache(PyObject*, PyObject* const* a, Py_ssize_t n) {
   for (int i = 0; i < n_written; ++i)
     for (int j = i + 1; j < n_spans; ++j)
       if (spans[i].lo < spans[j].hi && spans[j].lo < spans[i].hi) return none();
-  at::Tensor o = at::empty(q->sizes(), q->options());
-  at::Tensor lse = a[11] == Py_True ? rows_f32(*q) : at::Tensor();
-  if (!is_real(o) || (lse.defined() && !is_real(lse)) || (ws.defined() && !is_real(ws)))
-    return none();
-  void* w = ws.defined() ? ws.mutable_data_ptr() : nullptr;
-  float* l = lse.defined() ? static_cast<float*>(lse.mutable_data_ptr()) : nullptr;
+  const void *pq = q->const_data_ptr(), *pkn = kn->const_data_ptr(), *pvn = vn->const_data_ptr();
+  const void *pks = ks ? ks->const_data_ptr() : nullptr, *pvs = vs ? vs->const_data_ptr() : nullptr;
+  // (a commit writes the ring; without one it is only read)
+  void* const pkc = commit ? kc->mutable_data_ptr() : const_cast<void*>(kc->const_data_ptr());
+  void* const pvc = commit ? vc->mutable_data_ptr() : const_cast<void*>(vc->const_data_ptr());
   const int cap = static_cast<int>(kc->size(2));
-  const mw_status s = call([&] {
+  const bool need_lse = a[11] == Py_True;
+  const bool use_given = bytes > 0 && given && given->nbytes() >= bytes;
+  void* const pgiven = use_given ? given->mutable_data_ptr() : nullptr;
+  at::Tensor ws, o, lse;
+  mw_status s = MW_OK;
+  const bool real = call([&] {
+    if (bytes > 0 && !use_given) ws = scratch(bytes, options);
+    o = at::empty(sh, options);
+    if (need_lse) lse = rows_f32(sh, options);
+    if (!is_real(o) || (need_lse && !is_real(lse)) || (ws.defined() && !is_real(ws))) return false;
+    void* w = ws.defined() ? ws.mutable_data_ptr() : pgiven;
+    float* l = need_lse ? static_cast<float*>(lse.mutable_data_ptr()) : nullptr;
     cudaStream_t st = c10::cuda::getCurrentCUDAStream(dev).stream();
     if (commit)
-      return p_step(q->const_data_ptr(), kn->const_data_ptr(), vn->const_data_ptr(),
-                    kc->mutable_data_ptr(), vc->mutable_data_ptr(), cap, head, len, slot, rows,
-                    o.mutable_data_ptr(), l, w, bytes, B, H, W, T, d, scale, st);
-    return p_cache(q->const_data_ptr(), kn->const_data_ptr(), vn->const_data_ptr(),
-                   ks ? ks->const_data_ptr() : nullptr, vs ? vs->const_data_ptr() : nullptr,
-                   sink_len, kc->const_data_ptr(), vc->const_data_ptr(), cap, head, len, rope_dims,
-                   base, shift, o.mutable_data_ptr(), l, w, bytes, B, H, W, T, d, scale, st);
+      s = p_step(pq, pkn, pvn, pkc, pvc, cap, head, len, slot, rows, o.mutable_data_ptr(), l, w,
+                 bytes, B, H, W, T, d, scale, st);
+    else
+      s = p_cache(pq, pkn, pvn, pks, pvs, sink_len, pkc, pvc, cap, head, len, rope_dims, base,
+                  shift, o.mutable_data_ptr(), l, w, bytes, B, H, W, T, d, scale, st);
+    return true;
   });
+  if (!real) return none();
   if (s != MW_OK) return PyLong_FromLong(s);
   return result({&o, &lse});
   END_HANDLE_TH_ERRORS
@@ -345,16 +377,21 @@ PyObject* qkv(PyObject*, PyObject* const* a, Py_ssize_t n) {
       !real_number(a[2], &base) || !small_int(a[3], &per_frame) || !small_int(a[4], &first))
     return none();
   const int64_t B = x->size(0), N = x->size(1), H = x->size(3), d = x->size(4);
-  at::Tensor q = at::empty({B, H, N, d}, x->options());
-  at::Tensor k = at::empty({B, H, N, d}, x->options());
-  at::Tensor v = at::empty({B, H, N, d}, x->options());
-  if (!is_real(q) || !is_real(k) || !is_real(v)) return none();
-  const mw_status s = call([&] {
-    return p_qkv(x->const_data_ptr(), q.mutable_data_ptr(), k.mutable_data_ptr(),
-                 v.mutable_data_ptr(), static_cast<int>(B), static_cast<int>(N),
-                 static_cast<int>(H), static_cast<int>(d), dims, base, per_frame, first,
-                 c10::cuda::getCurrentCUDAStream(dev).stream());
+  const at::TensorOptions options = x->options();
+  const void* px = x->const_data_ptr();
+  at::Tensor q, k, v;
+  mw_status s = MW_OK;
+  const bool real = call([&] {
+    q = at::empty({B, H, N, d}, options);
+    k = at::empty({B, H, N, d}, options);
+    v = at::empty({B, H, N, d}, options);
+    if (!is_real(q) || !is_real(k) || !is_real(v)) return false;
+    s = p_qkv(px, q.mutable_data_ptr(), k.mutable_data_ptr(), v.mutable_data_ptr(),
+              static_cast<int>(B), static_cast<int>(N), static_cast<int>(H), static_cast<int>(d),
+              dims, base, per_frame, first, c10::cuda::getCurrentCUDAStream(dev).stream());
+    return true;
   });
+  if (!real) return none();
   if (s != MW_OK) return PyLong_FromLong(s);
   return result({&q, &k, &v});
   END_HANDLE_TH_ERRORS
