@@ -30,7 +30,7 @@ thread_local std::string g_last_error;
 // shared memory).  One per device: a static device variable.
 __device__ unsigned g_status_word;
 
-constexpr int kMaxDevices = 64;
+using mw::kMaxDevices;
 unsigned* g_status_ptr[kMaxDevices] = {};
 std::mutex g_mutex;
 

@@ -869,19 +869,18 @@ cudaError_t launch_bwd_main_t(const CUtensorMap& tq, const CUtensorMap& tk, cons
                               const CUtensorMap& tdo, const CUtensorMap& tdq,
                               const CUtensorMap& tbias, const BwdParams& p, cudaStream_t s) {
   using L = BwdLayout<D, DM>;
-  static bool attr_set = false;
-  if (!attr_set) {
+  static OncePerDevice prepared;
+  const cudaError_t e = prepared([] {
     // The in-kernel register re-split assumes the launch register count; with
     // any other count its setmaxnreg.inc could never be satisfied, so refuse.
     cudaFuncAttributes fa;
-    cudaError_t e0 = cudaFuncGetAttributes(&fa, bca_bwd_kernel<D, DM>);
+    const cudaError_t e0 = cudaFuncGetAttributes(&fa, bca_bwd_kernel<D, DM>);
     if (e0 != cudaSuccess) return e0;
     if (fa.numRegs != L::REGS_LAUNCH) return cudaErrorInvalidKernelImage;
-    cudaError_t e = cudaFuncSetAttribute(bca_bwd_kernel<D, DM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, L::BYTES);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+    return cudaFuncSetAttribute(bca_bwd_kernel<D, DM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                L::BYTES);
+  });
+  if (e != cudaSuccess) return e;
   const unsigned grid = static_cast<unsigned>(p.BH) * (p.N_pad / kTileRows);
   bca_bwd_kernel<D, DM><<<grid, L::THREADS, L::BYTES, s>>>(tq, tk, tv, tdo, tdq, tbias, p);
   return cudaGetLastError();

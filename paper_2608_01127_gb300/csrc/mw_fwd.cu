@@ -939,19 +939,18 @@ cudaError_t launch_fwd_t(const CUtensorMap& tq, const CUtensorMap& tk, const CUt
                          const CUtensorMap& tvs, const CUtensorMap& top, const FwdParams& p,
                          const RopeFreq& om, cudaStream_t s) {
   using L = FwdLayout<D, DM, ROPE, SPLIT>;
-  static bool attr_set = false;  // per process; the attribute is per function
-  if (!attr_set) {
+  static OncePerDevice prepared;
+  const cudaError_t e = prepared([] {
     // The in-kernel register re-split assumes the launch register count; with
     // any other count its setmaxnreg.inc could never be satisfied, so refuse.
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, bca_fwd_kernel<D, DM, ROPE, SPLIT>);
-    if (e != cudaSuccess) return e;
+    const cudaError_t e0 = cudaFuncGetAttributes(&fa, bca_fwd_kernel<D, DM, ROPE, SPLIT>);
+    if (e0 != cudaSuccess) return e0;
     if (fa.numRegs != L::REGS_LAUNCH) return cudaErrorInvalidKernelImage;
-    e = cudaFuncSetAttribute(bca_fwd_kernel<D, DM, ROPE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             L::BYTES);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+    return cudaFuncSetAttribute(bca_fwd_kernel<D, DM, ROPE, SPLIT>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, L::BYTES);
+  });
+  if (e != cudaSuccess) return e;
   const unsigned grid = static_cast<unsigned>(p.BH) * p.n_qblocks * p.num_splits;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace mw {
 
 // Rows of one query tile / key tile (the tcgen05 M and N of S = Q K^T).
@@ -123,6 +125,29 @@ inline void pdl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, dim3 
   cfg.attrs = &attr;
   cfg.numAttrs = g_pdl_enabled ? 1 : 0;
 }
+
+constexpr int kMaxDevices = 64;
+
+// Runs a kernel's setup once on each device: a function's attributes (its
+// dynamic shared memory) hold on the device that is current when they are set.
+// Threads may run it side by side; a setup that fails is tried again.
+class OncePerDevice {
+ public:
+  template <class F>
+  cudaError_t operator()(F&& setup) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (done_[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    e = setup();
+    if (e == cudaSuccess) done_[dev].store(true, std::memory_order_release);
+    return e;
+  }
+
+ private:
+  std::atomic<bool> done_[kMaxDevices] = {};
+};
 
 // Launchers (return cudaGetLastError() of the launch).
 // tkr/tvr: ring buffer maps; tks/tvs: sink anchor maps (any valid map when
