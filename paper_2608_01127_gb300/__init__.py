@@ -24,6 +24,8 @@ import importlib.machinery
 import importlib.util
 import math
 import os
+import sys
+import warnings
 from typing import Optional, Tuple
 
 import torch
@@ -133,6 +135,14 @@ def _load_native(lib: ctypes.CDLL) -> None:
             importlib.util.spec_from_loader("_mw_torch", loader))
         loader.exec_module(module)
     except ImportError:  # built against another PyTorch
+        return
+    # it reads PyTorch's objects through the headers it was built with
+    built = getattr(module, "torch_version", None), getattr(module, "python_hexversion", 0)
+    running = str(torch.__version__), sys.hexversion
+    if built != running:
+        warnings.warn(f"{_native_path} was built for PyTorch {built[0]} and Python {built[1]:#x}, "
+                      f"not PyTorch {running[0]} and Python {running[1]:#x}: it is not used, small "
+                      "calls take longer; build again", RuntimeWarning, stacklevel=3)
         return
     module.bind(*(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in (
         "mw_bca_fwd", "mw_bca_bwd", "mw_bca_bwd_workspace_size", "mw_bca_cache_workspace_size",

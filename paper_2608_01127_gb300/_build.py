@@ -48,6 +48,7 @@ def _torch_module() -> list:
     lib = os.path.join(root, "lib")
     return [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared",
             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            f'-DMW_TORCH_VERSION="{torch.__version__}"',
             "-I" + INCLUDE, "-isystem", os.path.join(root, "include"),
             "-isystem", sysconfig.get_paths()["include"],
             "-isystem", os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"),

@@ -410,4 +410,14 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_mw_torch", nullptr, -1, methods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__mw_torch(void) { return PyModule_Create(&module); }
+// The PyTorch and Python it was built for: it reads their objects' fields through
+// their headers, and another version's symbols may resolve all the same.
+PyMODINIT_FUNC PyInit__mw_torch(void) {
+  PyObject* m = PyModule_Create(&module);
+  if (m && (PyModule_AddStringConstant(m, "torch_version", MW_TORCH_VERSION) < 0 ||
+            PyModule_AddIntConstant(m, "python_hexversion", PY_VERSION_HEX) < 0)) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}
