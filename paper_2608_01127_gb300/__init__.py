@@ -120,30 +120,33 @@ def library() -> ctypes.CDLL:
         fn = getattr(lib, name)
         fn.restype = res
         fn.argtypes = args
-    _load_native(lib)
     _lib = lib
+    _load_native(lib)
     return lib
 
 
 def _load_native(lib: ctypes.CDLL) -> None:
     global _native
+
+    def without(why: str) -> None:
+        warnings.warn(f"{_native_path} {why}: calls go the longer way, two to three times as long "
+                      "for small ones; build again", RuntimeWarning, stacklevel=4)
+
     if not os.path.exists(_native_path):
-        return
+        return without("is missing")
     loader = importlib.machinery.ExtensionFileLoader("_mw_torch", _native_path)
     try:
         module = importlib.util.module_from_spec(
             importlib.util.spec_from_loader("_mw_torch", loader))
         loader.exec_module(module)
-    except ImportError:  # built against another PyTorch
-        return
+    except ImportError as e:
+        return without(f"was not loaded ({e})")
     # it reads PyTorch's objects through the headers it was built with
     built = getattr(module, "torch_version", None), getattr(module, "python_hexversion", 0)
     running = str(torch.__version__), sys.hexversion
     if built != running:
-        warnings.warn(f"{_native_path} was built for PyTorch {built[0]} and Python {built[1]:#x}, "
-                      f"not PyTorch {running[0]} and Python {running[1]:#x}: it is not used, small "
-                      "calls take longer; build again", RuntimeWarning, stacklevel=3)
-        return
+        return without(f"was built for PyTorch {built[0]} and Python {built[1]:#x}, not PyTorch "
+                       f"{running[0]} and Python {running[1]:#x}")
     module.bind(*(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in (
         "mw_bca_fwd", "mw_bca_bwd", "mw_bca_bwd_workspace_size", "mw_bca_cache_workspace_size",
         "mw_bca_cache_fwd_rope", "mw_bca_cache_step", "mw_qkv_rope_split")))
