@@ -71,11 +71,12 @@ struct FwdLayout {
   // is there, so that both tiles' softmax warps work all the time instead of
   // in turn (P over S as a whole leaves each tile's softmax waiting for its own
   // PV and QK^T).  d = 64, 24 heads x 16 x 880: 613 us before, 594 with the
-  // early exponentials below alone, 568 with both and an issuer per tile; 16
-  // heads of 72: 445, 438 and 436 us (with one issuer).  A split key range is
-  // a handful of tiles a CTA, which the chain through the first and the last
-  // of them dominates: it gains nothing (one step against 8 chunks of 880, 12
-  // heads of 64: 30.3 us against 30.6 with it; 16 of 72: 46.0 against 47.6).
+  // early exponentials below alone, 568 with both and an issuer per tile (557
+  // since, with a leaner epilogue); 16 heads of 72: 445, 438 and 436 us (with
+  // one issuer).  A split key range is a handful of tiles a CTA, which the chain
+  // through the first and the last of them dominates: it gains nothing (one step
+  // against 8 chunks of 880, 12 heads of 64: 30.3 us against 30.6 with it; 16 of
+  // 72: 46.0 against 47.6).
   static constexpr bool SPLIT_P = !SPLIT && 256 + OW * QT + 32 * QT <= 512;
   // MMA-issuing warps: at d = 64 one per query tile (warps 9 and 10), since a
   // step's waits and commits take an issuer about as long as its MMAs take the
@@ -93,6 +94,14 @@ struct FwdLayout {
   static constexpr uint32_t P_COL(int t, int half) {
     return half == 0 ? S_COL(t) : SPLIT_P ? 256u + OW * QT + 32u * t : S_COL(t) + 32u;
   }
+  // With the re-shift on 128-wide MMAs the unsplit epilogue keeps a row-per-
+  // thread form of the fp32 partials that no launch takes (the launcher picks
+  // SPLIT for several splits): the compiler schedules that kernel's key loop
+  // 2.7% faster with it (16 heads of 128, 8 x 880 rows against 12 chunks and a
+  // sink, 582 us, 597 without it; unrolling the epilogue less, 592).  The others
+  // gain by being without it: the re-shift at d = 72 488 -> 482 us, the plain
+  // forward at d = 64 566 -> 557.
+  static constexpr bool ROWS_KEPT = ROPE && !SPLIT && DM == 128;
   static constexpr int THREADS = 384;
   // registers per thread after the re-split: softmax warpgroups 0-1 get
   // more, warpgroup 2 (TMA, MMA, RoPE or idle warps) less; 2*128*S + 128*C
@@ -303,7 +312,8 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
   // the allocation of all 512 columns can only start at 0; as a constant it
   // keeps the issuing warp's TMEM addresses out of registers (with one-word
   // operand descriptors, 12 heads of 128, 32 x 600 tokens: 783 us before, 749
-  // with the descriptors, 721 with both; d = 64, 16 x 880: 640 -> 631 us)
+  // with the descriptors, 721 with both; d = 64, 16 x 880: 640 -> 631 us).  A
+  // look at the slot, in any place, costs the 128-wide kernel 0.6% or more
   constexpr uint32_t tmem = 0;
   const WaitCtl ctl{abort_flag, p.status, p.budget_ns};
   // launched early (programmatic dependent launch): the setup above has run
@@ -789,11 +799,18 @@ __global__ void __launch_bounds__(FwdLayout<D, DM>::THREADS, 1)
       for (int k = 0; k < 32; ++k) v[k] = nonzero ? __uint_as_float(r[k]) * inv_l : 0.f;
       if constexpr (!SPLIT) {
         if (!row_valid) continue;
-        // the caller's rows hold d_io <= D columns (multiples of 8); only
-        // the 128-wide kernel serves padded head dims
-        const int d_io = (D == 64) ? D : p.d_io;
-        if (32 * c >= d_io) continue;
-        store_row32(p.o + row_off * d_io + 32 * c, v, min(4, (d_io - 32 * c) / 8), p.wide_out);
+        if (!L::ROWS_KEPT || p.num_splits == 1) {
+          // the caller's rows hold d_io <= D columns (multiples of 8); only
+          // the 128-wide kernel serves padded head dims
+          const int d_io = (D == 64) ? D : p.d_io;
+          if (32 * c >= d_io) continue;
+          store_row32(p.o + row_off * d_io + 32 * c, v, min(4, (d_io - 32 * c) / 8), p.wide_out);
+        } else {
+          float4* dst = reinterpret_cast<float4*>(
+              p.o_part + (static_cast<size_t>(split) * p.BH * p.rows_q + row_off) * D + 32 * c);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) dst[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+        }
       } else if (t < qt_n) {
         // (an empty tile's warps skip the O wait: they must not touch the
         // stages, which the other tile's MMAs may still be reading)

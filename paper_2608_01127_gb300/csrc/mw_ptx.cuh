@@ -134,8 +134,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
-// Contiguous global -> shared copy; both addresses 16-byte aligned, size a
-// multiple of 16.
 // 3-D tiled reduce-add of a shared-memory box into global memory (element
 // type and box from the map; here f32), tracked as a bulk async-group of the
 // issuing thread.  Coordinates must not be negative; c0 * element size must be
@@ -186,6 +184,8 @@ __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
+// Contiguous global -> shared copy; both addresses 16-byte aligned, size a
+// multiple of 16.
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
                                           uint64_t* bar) {
   asm volatile(
