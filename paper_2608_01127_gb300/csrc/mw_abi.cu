@@ -182,15 +182,13 @@ mw_status make_map(CUtensorMap* m, const void* ptr, int rows, int BH, int d, con
   return MW_OK;
 }
 
-mw_status status_ptr(unsigned** out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return fail(MW_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
+// (dev: the current device)
+mw_status status_ptr(int dev, unsigned** out) {
   if (dev < 0 || dev >= kMaxDevices) return fail(MW_ERR_CUDA, "device index %d too large", dev);
   std::lock_guard<std::mutex> lock(g_mutex);
   if (!g_status_ptr[dev]) {
     void* p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_status_word);
+    const cudaError_t e = cudaGetSymbolAddress(&p, g_status_word);
     if (e != cudaSuccess) return fail(MW_ERR_CUDA, "cudaGetSymbolAddress: %s", cudaGetErrorString(e));
     g_status_ptr[dev] = static_cast<unsigned*>(p);
   }
@@ -385,6 +383,7 @@ class DeviceScope {
     if (err_ != cudaSuccess) return fail(MW_ERR_CUDA, "cudaSetDevice: %s", cudaGetErrorString(err_));
     return MW_OK;
   }
+  int device() const { return dev_; }
 
  private:
   int prev_ = -1, dev_ = 0;
@@ -421,7 +420,7 @@ mw_status fwd_common(const void* q, const void* k, const void* v, const void* kr
   DeviceScope scope(stream);
   MW_TRY(scope.status());
   unsigned* status = nullptr;
-  MW_TRY(status_ptr(&status));
+  MW_TRY(status_ptr(scope.device(), &status));
   CUtensorMap tq, tk, tv, tkr, tvr, tks, tvs;
   MW_TRY(make_map(&tq, q, rows_q, BH, d, "q"));
   MW_TRY(make_map(&tk, k, rows_q, BH, d, "k"));
@@ -485,7 +484,7 @@ mw_status fwd_common(const void* q, const void* k, const void* v, const void* kr
     MW_TRY(make_map(&top, p.o_part, rows_q, p.num_splits * BH, D, "o_part", mw::kTileRows, true));
   }
   MW_TRY(launch_status(mw::launch_fwd(D, mma_d(d), tq, tk, tv, tkr, tvr, tks, tvs, top, p, rope.omega,
-                                      stream),
+                                      scope.device(), stream),
                        "forward kernel launch"));
   if (p.num_splits > 1)
     MW_TRY(launch_status(mw::launch_combine(D, d, p.o_part, p.lse_part, p.o, lse, p.num_splits, BH,
@@ -630,7 +629,7 @@ mw_status mw_bca_bwd_stage(int stage, const void* q, const void* k, const void* 
                          "backward pre kernel launch"));
   if (main) {
     unsigned* status = nullptr;
-    MW_TRY(status_ptr(&status));
+    MW_TRY(status_ptr(scope.device(), &status));
     CUtensorMap tq, tk, tv, tdo, tdq;
     const int D = kernel_d(d);
     const int qrows = mw::bwd_q_rows(D);  // query rows per backward step
@@ -659,7 +658,7 @@ mw_status mw_bca_bwd_stage(int stage, const void* q, const void* k, const void* 
     p.status = status;
     p.budget_ns = budget_ns();
     p.debug_skip_q = static_cast<int>(g_opt_skip_q);
-    MW_TRY(launch_status(mw::launch_bwd_main(D, mma_d(d), tq, tk, tv, tdo, tdq, tbias, p, s),
+    MW_TRY(launch_status(mw::launch_bwd_main(D, mma_d(d), tq, tk, tv, tdo, tdq, tbias, p, scope.device(), s),
                          "backward kernel launch"));
   }
   if (post)
@@ -894,7 +893,7 @@ mw_status mw_device_status(void* stream, int clear) {
   DeviceScope scope(s);
   MW_TRY(scope.status());
   unsigned* ptr = nullptr;
-  MW_TRY(status_ptr(&ptr));
+  MW_TRY(status_ptr(scope.device(), &ptr));
   cudaError_t e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(MW_ERR_CUDA, "cudaStreamSynchronize: %s", cudaGetErrorString(e));
   unsigned word = 0;

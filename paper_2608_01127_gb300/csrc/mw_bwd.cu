@@ -867,10 +867,10 @@ __global__ void __launch_bounds__(256) bwd_post_kernel(const float* __restrict__
 template <int D, int DM>
 cudaError_t launch_bwd_main_t(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                               const CUtensorMap& tdo, const CUtensorMap& tdq,
-                              const CUtensorMap& tbias, const BwdParams& p, cudaStream_t s) {
+                              const CUtensorMap& tbias, const BwdParams& p, int dev, cudaStream_t s) {
   using L = BwdLayout<D, DM>;
   static OncePerDevice prepared;
-  const cudaError_t e = prepared([] {
+  const cudaError_t e = prepared(dev, [] {
     // The in-kernel register re-split assumes the launch register count; with
     // any other count its setmaxnreg.inc could never be satisfied, so refuse.
     cudaFuncAttributes fa;
@@ -902,10 +902,10 @@ cudaError_t launch_bwd_pre(int d, int d_io, const __nv_bfloat16* o, const __nv_b
 
 cudaError_t launch_bwd_main(int d, int dm, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const CUtensorMap& tdo, const CUtensorMap& tdq,
-                            const CUtensorMap& tbias, const BwdParams& p, cudaStream_t s) {
-  if (d == 64) return launch_bwd_main_t<64, 64>(tq, tk, tv, tdo, tdq, tbias, p, s);
-  if (dm == 80) return launch_bwd_main_t<128, 80>(tq, tk, tv, tdo, tdq, tbias, p, s);
-  return launch_bwd_main_t<128, 128>(tq, tk, tv, tdo, tdq, tbias, p, s);
+                            const CUtensorMap& tbias, const BwdParams& p, int dev, cudaStream_t s) {
+  if (d == 64) return launch_bwd_main_t<64, 64>(tq, tk, tv, tdo, tdq, tbias, p, dev, s);
+  if (dm == 80) return launch_bwd_main_t<128, 80>(tq, tk, tv, tdo, tdq, tbias, p, dev, s);
+  return launch_bwd_main_t<128, 128>(tq, tk, tv, tdo, tdq, tbias, p, dev, s);
 }
 
 cudaError_t launch_bwd_post(int d, int d_io, const float* dq_acc, __nv_bfloat16* dq, float scale,

@@ -954,10 +954,10 @@ template <int D, int DM, bool ROPE, bool SPLIT>
 cudaError_t launch_fwd_t(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                          const CUtensorMap& tkr, const CUtensorMap& tvr, const CUtensorMap& tks,
                          const CUtensorMap& tvs, const CUtensorMap& top, const FwdParams& p,
-                         const RopeFreq& om, cudaStream_t s) {
+                         const RopeFreq& om, int dev, cudaStream_t s) {
   using L = FwdLayout<D, DM, ROPE, SPLIT>;
   static OncePerDevice prepared;
-  const cudaError_t e = prepared([] {
+  const cudaError_t e = prepared(dev, [] {
     // The in-kernel register re-split assumes the launch register count; with
     // any other count its setmaxnreg.inc could never be satisfied, so refuse.
     cudaFuncAttributes fa;
@@ -980,15 +980,15 @@ template <bool SPLIT>
 cudaError_t launch_fwd_split(int d, int dm, const CUtensorMap& tq, const CUtensorMap& tk,
                              const CUtensorMap& tv, const CUtensorMap& tkr, const CUtensorMap& tvr,
                              const CUtensorMap& tks, const CUtensorMap& tvs, const CUtensorMap& top,
-                             const FwdParams& p, const RopeFreq& om, cudaStream_t s) {
+                             const FwdParams& p, const RopeFreq& om, int dev, cudaStream_t s) {
   if (p.rope_dims > 0) {
-    if (d == 64) return launch_fwd_t<64, 64, true, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
-    if (dm == 80) return launch_fwd_t<128, 80, true, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
-    return launch_fwd_t<128, 128, true, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
+    if (d == 64) return launch_fwd_t<64, 64, true, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
+    if (dm == 80) return launch_fwd_t<128, 80, true, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
+    return launch_fwd_t<128, 128, true, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
   }
-  if (d == 64) return launch_fwd_t<64, 64, false, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
-  if (dm == 80) return launch_fwd_t<128, 80, false, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
-  return launch_fwd_t<128, 128, false, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
+  if (d == 64) return launch_fwd_t<64, 64, false, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
+  if (dm == 80) return launch_fwd_t<128, 80, false, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
+  return launch_fwd_t<128, 128, false, SPLIT>(tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
 }
 
 }  // namespace
@@ -996,9 +996,9 @@ cudaError_t launch_fwd_split(int d, int dm, const CUtensorMap& tq, const CUtenso
 cudaError_t launch_fwd(int d, int dm, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                        const CUtensorMap& tkr, const CUtensorMap& tvr, const CUtensorMap& tks,
                        const CUtensorMap& tvs, const CUtensorMap& top, const FwdParams& p,
-                       const RopeFreq& om, cudaStream_t s) {
-  return p.num_splits > 1 ? launch_fwd_split<true>(d, dm, tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s)
-                          : launch_fwd_split<false>(d, dm, tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, s);
+                       const RopeFreq& om, int dev, cudaStream_t s) {
+  return p.num_splits > 1 ? launch_fwd_split<true>(d, dm, tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s)
+                          : launch_fwd_split<false>(d, dm, tq, tk, tv, tkr, tvr, tks, tvs, top, p, om, dev, s);
 }
 
 cudaError_t launch_combine(int d, int d_io, const float* o_part, const float* lse_part,

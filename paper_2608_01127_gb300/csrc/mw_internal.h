@@ -133,14 +133,12 @@ constexpr int kMaxDevices = 64;
 // Threads may run it side by side; a setup that fails is tried again.
 class OncePerDevice {
  public:
+  // dev: the current device
   template <class F>
-  cudaError_t operator()(F&& setup) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
+  cudaError_t operator()(int dev, F&& setup) {
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (done_[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    e = setup();
+    const cudaError_t e = setup();
     if (e == cudaSuccess) done_[dev].store(true, std::memory_order_release);
     return e;
   }
@@ -149,7 +147,7 @@ class OncePerDevice {
   std::atomic<bool> done_[kMaxDevices] = {};
 };
 
-// Launchers (return cudaGetLastError() of the launch).
+// Launchers (return cudaGetLastError() of the launch; dev: the current device).
 // tkr/tvr: ring buffer maps; tks/tvs: sink anchor maps (any valid map when
 // the segment is empty)
 // d: tile width (64 or 128); dm: MMA width (d, or 80 on the 128-wide tiles
@@ -159,7 +157,7 @@ class OncePerDevice {
 cudaError_t launch_fwd(int d, int dm, const CUtensorMap& tq, const CUtensorMap& tk,
                        const CUtensorMap& tv, const CUtensorMap& tkr, const CUtensorMap& tvr, const CUtensorMap& tks,
                        const CUtensorMap& tvs, const CUtensorMap& top, const FwdParams& p,
-                       const RopeFreq& rope_om, cudaStream_t s);
+                       const RopeFreq& rope_om, int dev, cudaStream_t s);
 // d: the kernels' head dim (64 or 128); d_io: the caller's (a multiple of 8, <= d)
 // The combine's launch also carries the ring commit `cj` (if cj.rows > 0)
 // in blocks of its own: both only run once the forward has finished, and
@@ -180,7 +178,7 @@ cudaError_t launch_bwd_pre(int d, int d_io, const __nv_bfloat16* o, const __nv_b
 // 32-byte swizzle (d = 128: any map, unused)
 cudaError_t launch_bwd_main(int d, int dm, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const CUtensorMap& tdo, const CUtensorMap& tdq,
-                            const CUtensorMap& tbias, const BwdParams& p, cudaStream_t s);
+                            const CUtensorMap& tbias, const BwdParams& p, int dev, cudaStream_t s);
 cudaError_t launch_bwd_post(int d, int d_io, const float* dq_acc, __nv_bfloat16* dq, float scale,
                             int BH, int N, int N_pad, cudaStream_t s);
 // d: any multiple of 8 (rows are copied in 16-byte pieces)
